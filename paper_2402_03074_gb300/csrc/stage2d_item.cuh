@@ -13,6 +13,7 @@
 // two ring columns per band and the two ring rows per chunk (x pass skipped on ring rows).
 #pragma once
 #include "hweno_device.cuh"
+#include "stage2d_char64.cuh"
 
 namespace hw {
 
@@ -59,32 +60,30 @@ __device__ __forceinline__ void volume_sum(const KProblem& P, int dir, const R (
 // The row window holds the stage input in the bulk precision R (converted once per value
 // when a row is loaded); the FP64 update reads the cell's own averages from global memory
 // when R is float.
-//
-// Characteristic FP64 Euler in 96-thread blocks (kCoefOnce): the Appendix coefficients of p_0
-// are linear in the stencil and the projection L is linear, so the coefficients of a field's
-// p_0 are L applied to the coefficient vectors of the conserved components.  Those are formed
-// once per cell for both passes (4 x 64 operations, kept in shared memory: 60 values per
-// thread) and each pass projects the 15 coefficient vectors instead of forming 4 x 15
-// coefficients from 17 projected stencil vectors: 188 fewer FP64 operations per cell.  The
-// extra 46 KB per block fit two blocks per SM at 96 threads (109 KB each), not at 128 (145 KB).
-template <int EQ, bool CHAR, typename R, int BW>
-constexpr bool kCoefOnce = EQ == EQ_EULER && CHAR && sizeof(R) == sizeof(double) && BW == 96;
 
-// Shared memory of a block: the 3-row window, the x-face exchange, the top traces carried
+// Characteristic FP64 Euler has an item of its own (stage2d_char64.cuh).
+template <int EQ, bool CHAR, typename R>
+constexpr bool kChar64 = EQ == EQ_EULER && CHAR && sizeof(R) == sizeof(double);
+
+// Shared memory of a block: the 3-row window, the x-face exchange and the top traces carried
 // from row to row (in shared memory rather than in 48 registers: fewer spills, FP32-bulk
-// stages 2 % faster) and (kCoefOnce) the conserved coefficients.
+// stages 2 % faster).
 template <int EQ, bool CHAR, typename R, int BW>
 constexpr size_t smem_bytes2d() {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
+  if constexpr (kChar64<EQ, CHAR, R>) return smem_bytes_char64<BW>();
   return sizeof(R) * 3 * NC * 3 * (BW + 2) + sizeof(R) * NC * 3 * 2 * BW +
-         sizeof(R) * 2 * 3 * NC * BW +
-         (kCoefOnce<EQ, CHAR, R, BW> ? sizeof(R) * NC * 15 * BW : 0);
+         sizeof(R) * 2 * 3 * NC * BW;
 }
 
 template <int EQ, bool CHAR, typename R, int BW>
 __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S, int band,
                                              int j0, int j1, int wout, double* smem,
                                              double (*red)[BW / 32]) {
+  if constexpr (kChar64<EQ, CHAR, R>) {
+    stage2d_char64_item<BW>(P, S, band, j0, j1, wout, smem, red);
+    return;
+  }
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
   constexpr int NM = 3;
   constexpr int NA = NC * NM;
@@ -102,10 +101,6 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
   R* car = trL + NC * 3 * 2 * BW;
   auto prevT = [&](int g, int c) -> R& { return car[((0 * 3 + g) * NC + c) * BW + threadIdx.x]; };
   auto prevTg = [&](int g, int c) -> R& { return car[((1 * 3 + g) * NC + c) * BW + threadIdx.x]; };
-  // kCoefOnce: the Appendix coefficients of the conserved components of the thread's cell,
-  // [component][15][BW] (each thread reads only its own column)
-  R* cco = car + 2 * 3 * NC * BW;
-  (void)cco;
 
   const int nx = P.nx, ny = P.ny;
   const size_t plane = (size_t)nx * ny;
@@ -214,22 +209,6 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
 #pragma unroll
         for (int c = 0; c < 4; ++c) U5[c] = Wv(c * NM, 4);
         E.init_state(P, U5);
-        if constexpr (kCoefOnce<EQ, CHAR, R, BW>) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            R u[9], v[4], w[4], cf[15];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) u[k] = Wv(c * NM, k);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              v[e] = Wv(c * NM + 1, 2 * e + 1);
-              w[e] = Wv(c * NM + 2, 2 * e + 1);
-            }
-            coeffs2d<R>(u, v, w, cf);
-#pragma unroll
-            for (int n = 0; n < 15; ++n) cco[(c * 15 + n) * BW + t] = cf[n];
-          }
-        }
       }
 #pragma unroll
       for (int pass = 0; pass < 2; ++pass) {
@@ -255,44 +234,7 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
 #pragma unroll
             for (int p = 0; p < 9; ++p) ch[6 + p][f] = in[p];
           };
-          if constexpr (kCoefOnce<EQ, CHAR, R, BW>) {
-            // the shared projection terms of the 15 coefficient vectors, and the averages of
-            // cells 2, 4, 5, 6, 8 (u_ave, the linear polynomials) in characteristic variables
-            const int tang = pass == 0 ? 2 : 1;  // tangential momentum component
-            R cs[15], ct[15];
-#pragma unroll
-            for (int n = 0; n < 15; ++n) {
-              R Uc[4];
-#pragma unroll
-              for (int c = 0; c < 4; ++c) Uc[c] = cco[(c * 15 + n) * BW + t];
-              E.shared_terms(Uc, cs[n], ct[n]);
-            }
-            R Wa[5][4];
-#pragma unroll
-            for (int e = 0; e < 5; ++e) {
-              const int k = e == 0 ? 1 : (e == 4 ? 7 : e + 2);  // cells 2, 4, 5, 6, 8
-              R Uk[4];
-#pragma unroll
-              for (int c = 0; c < 4; ++c) Uk[c] = Wv(c * NM, k);
-              E.project_all(Uk, Wa[e]);
-            }
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-              R cf[15], u[9], C[15];
-#pragma unroll
-              for (int n = 0; n < 15; ++n)
-                cf[n] = E.field_of(f, cs[n], ct[n], cco[n * BW + t],
-                                   cco[(tang * 15 + n) * BW + t]);
-              u[0] = u[2] = u[6] = u[8] = R(0);
-              u[1] = Wa[0][f];
-              u[3] = Wa[1][f];
-              u[4] = Wa[2][f];
-              u[5] = Wa[3][f];
-              u[7] = Wa[4][f];
-              recon2d_from_coeffs<R, 0>(cf, u, P, C, fast_weights);
-              evaluate(f, C);
-            }
-          } else {
+          {
             // the stencil in characteristic variables, all four fields at once: 9 averages
             // and the x / y first moments of cells 2, 4, 6, 8
             R Wu[9][4], Wv_[4][4], Ww[4][4];
@@ -325,46 +267,35 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
                 w[e] = Ww[e][f];
               }
             };
-            // field by field: coefficients, FP64 smoothness indicators and weights (the
-            // branch-free product form, the direct formula only where it does not apply),
-            // combination and evaluation.  The FP32-bulk class takes the fields in pairs whose
+            // per field: coefficients, FP64 smoothness indicators and weights (the branch-free
+            // product form), combination and evaluation.  The fields are taken in pairs whose
             // two FP64 weight chains share a basic block (the direct formula, for the rare
             // cells that need it, after both), which hides part of their latency: 9.10 ms
             // against 9.20-9.27 ms per 2048^2 stage
-            if constexpr (sizeof(R) == sizeof(double)) {
 #pragma unroll
-              for (int f = 0; f < 4; ++f) {
-                R u[9], v[4], w[4], C[15];
-                field(f, u, v, w);
-                recon2d_coeffs<R, 0>(u, v, w, P, C, fast_weights);
-                evaluate(f, C);
+            for (int f0 = 0; f0 < 4; f0 += 2) {
+              bool ok = true;
+              R C0[15], C1[15];
+              {
+                R u[9], v[4], w[4];
+                field(f0, u, v, w);
+                recon2d_coeffs<R, 1>(u, v, w, P, C0, ok);
               }
-            } else {
-#pragma unroll
-              for (int f0 = 0; f0 < 4; f0 += 2) {
-                bool ok = true;
-                R C0[15], C1[15];
-                {
-                  R u[9], v[4], w[4];
-                  field(f0, u, v, w);
-                  recon2d_coeffs<R, 1>(u, v, w, P, C0, ok);
-                }
-                {
-                  R u[9], v[4], w[4];
-                  field(f0 + 1, u, v, w);
-                  recon2d_coeffs<R, 1>(u, v, w, P, C1, ok);
-                }
-                if (!ok) {
-                  fast_weights = false;
-                  R u[9], v[4], w[4];
-                  field(f0, u, v, w);
-                  recon2d_coeffs<R, 2>(u, v, w, P, C0, ok);
-                  field(f0 + 1, u, v, w);
-                  recon2d_coeffs<R, 2>(u, v, w, P, C1, ok);
-                }
-                evaluate(f0, C0);
-                evaluate(f0 + 1, C1);
+              {
+                R u[9], v[4], w[4];
+                field(f0 + 1, u, v, w);
+                recon2d_coeffs<R, 1>(u, v, w, P, C1, ok);
               }
+              if (!ok) {
+                fast_weights = false;
+                R u[9], v[4], w[4];
+                field(f0, u, v, w);
+                recon2d_coeffs<R, 2>(u, v, w, P, C0, ok);
+                field(f0 + 1, u, v, w);
+                recon2d_coeffs<R, 2>(u, v, w, P, C1, ok);
+              }
+              evaluate(f0, C0);
+              evaluate(f0 + 1, C1);
             }
           }
           R cons[16][4];
