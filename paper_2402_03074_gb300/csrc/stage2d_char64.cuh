@@ -30,45 +30,130 @@ namespace c64 {
 constexpr double S1 = 0.38729833462074168852;  // sqrt(15)/10, the outer Gauss node
 constexpr double S2 = 0.15, S3 = S1 * 0.15, S4 = 0.0225;
 
+// The FP64 unit takes 16 clocks per warp for a DFMA whose three operands are vector registers
+// and 19 for a DADD, a DMUL or a DFMA with a constant or uniform operand (measured: 2.00 and
+// 1.68 lanes per clock and SM, whatever the number of warps).  So every operation here is a
+// three-register DFMA: a + b = a 1 + b, a b = a b + (-0), both exact, with 1 and -0 held in
+// registers, and the constants are read from shared memory into registers at each use, through
+// an address that depends on the thread (a provably uniform one would be loaded into a uniform
+// register).  2048^2 stage: 21.2 ms with plain operators, 18.8 ms so.
+#define HW_C64_CONSTANTS(X)                                                                   \
+  X(ONE, 1.0) X(NZERO, -0.0)                                                                  \
+  /* beta_0 */                                                                                \
+  X(B_A8, S1 / (12.0 * S3)) X(B_A6, S1 / (4.0 * S3)) X(B_W1, 1.0 / S2)                        \
+  X(B_W6, 781.0 / (20.0 * S3 * S3)) X(B_W8, 47.0 / (10.0 * S3 * S3))                          \
+  X(B_C12, S2 / (12.0 * S4)) X(B_C10, 63.0 * S2 / (130.0 * S4))                               \
+  X(B_W3, 13.0 / (3.0 * S2 * S2)) X(B_W10, 1421461.0 / (2275.0 * S4 * S4))                    \
+  X(B_W12, 5083.0 * 144.0 / (270.0 * S2 * S2)) X(B_E, 17.0 * S2 / (70.0 * S4))                \
+  X(B_W4, 7.0 / (6.0 * S2 * S2)) X(B_WP, 710728.0 / (33600.0 * S4 * S4))                      \
+  X(B_WM, 710730.0 / (33600.0 * S4 * S4))                                                     \
+  /* weights */                                                                               \
+  X(W_TAU, 25.0 / 16.0) X(MTWO, -2.0)                                                         \
+  /* evaluation */                                                                            \
+  X(M12, -25.0 / 81.0) X(MX, -5.0 / 9.0) X(V8, 1.0 / (144.0 * S3)) X(V6, 1.0 / (80.0 * S3))   \
+  X(V1, 1.0 / (12.0 * S1)) X(H1, 0.5 / S1) X(H2, 0.25 / S2) X(H3, 0.125 / S3)                 \
+  X(H4, 0.0625 / S4)                                                                          \
+  /* the Appendix coefficients */                                                             \
+  X(MFOUR, -4.0) X(A1X, S1 / 48.0) X(A1E, -397.0 / 456.0 * S1) X(A1V, -75.0 / 19.0 * S1)      \
+  X(A6E, 5.0 / 19.0 * S3) X(A6V, 60.0 / 19.0 * S3) X(A8X, -0.25 * S3) X(A8E, 0.5 * S3)        \
+  X(A4X, -7.0 / 22.0 * S2) X(A4V, 75.0 / 11.0 * S2) X(A11X, 5.0 / 22.0 * S4)                  \
+  X(A11V, -60.0 / 11.0 * S4) X(A3R, -S2 / 48.0) X(A3Q, S2 / 24.0) X(A3P, 71.0 / 48.0 * S2)    \
+  X(A3V, -45.0 / 8.0 * S2) X(A10P, -5.0 / 8.0 * S4) X(A10V, 15.0 / 4.0 * S4)                  \
+  X(A12R, 0.25 * S4) X(A12P, -0.5 * S4)                                                       \
+  /* cell, volume and faces */                                                                \
+  X(HALF, 0.5) X(WC, 25.0 / 324.0) X(WE, 10.0 / 81.0) X(WM, 16.0 / 81.0)                      \
+  X(THREEQ, 0.75) X(QUARTER, 0.25) X(THIRD, 1.0 / 3.0) X(TWOTHIRD, 2.0 / 3.0)
+enum Const : int {
+#define X(name, value) k##name,
+  HW_C64_CONSTANTS(X)
+#undef X
+  kStatic,             // from here on: values of the problem, written at the start of an item
+  kEPS = kStatic, kGLO, kG0, kSGLO, kGM1, kHGM1, kGAM, kIDX, kFX0, kFX1, kFX2, kFY0, kFY1, kFY2,
+  kIDY, kCount
+};
+static __constant__ double c64_constants[kStatic] = {
+#define X(name, value) (value),
+    HW_C64_CONSTANTS(X)
+#undef X
+};
+constexpr int kTable = (kCount + 7) / 8 * 8;  // doubles of shared memory
+
+struct Ops {
+  double one, nz;
+  unsigned tab;  // shared address of the table (+ 0 for every thread, which no pass can prove)
+  template <int I>
+  __device__ __forceinline__ double k() const {
+    double v;  // volatile: a constant is loaded where it is used, not kept in registers
+    asm volatile("ld.shared.f64 %0, [%1+%2];" : "=d"(v) : "r"(tab), "n"(8 * I));
+    return v;
+  }
+  __device__ __forceinline__ double add(double a, double b) const { return fma(a, one, b); }
+  __device__ __forceinline__ double sub(double a, double b) const { return fma(-b, one, a); }
+  __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, nz); }
+};
+#define K(name) o.k<k##name>()
+
+// the table of an item (visible after the caller's next __syncthreads)
+__device__ __forceinline__ void fill_table(double* tab, const KProblem& P) {
+  const int t = threadIdx.x;
+  static_assert(kStatic <= 64, "one entry per thread of the narrowest block");
+  if (t < kStatic) tab[t] = c64_constants[t];
+  if (t == 0) {
+    tab[kEPS] = 25.0 * P.eps;  // d_m is scaled by 25, the squared divisor of u_ave
+    tab[kGLO] = P.glo;
+    tab[kG0] = P.g0[1];
+    tab[kSGLO] = S1 * P.glo;
+    tab[kGM1] = P.gm1;
+    tab[kHGM1] = -0.5 * P.gm1;
+    tab[kGAM] = P.gam;
+    // Gauss moments of a face from twice its flux, divided by the cell size
+    tab[kIDX] = P.inv_dx;
+    tab[kFX0] = 5.0 / 36.0 * P.inv_dx;
+    tab[kFX1] = 2.0 / 9.0 * P.inv_dx;
+    tab[kFX2] = 5.0 / 36.0 * S1 * P.inv_dx;
+    tab[kIDY] = P.inv_dy;
+    tab[kFY0] = 5.0 / 36.0 * P.inv_dy;
+    tab[kFY1] = 2.0 / 9.0 * P.inv_dy;
+    tab[kFY2] = 5.0 / 36.0 * S1 * P.inv_dy;
+  }
+}
+
 // 1/x of a normal double with exponent field in [1, 2044]: the hardware's 20-bit reciprocal,
 // refined by one third-order step y + y (e + e^2), e = 1 - x y (the new residual e^3 < 2^-59).
-__device__ __forceinline__ double rcp_seed(double x) {
+__device__ __forceinline__ double rcp_in_range(const Ops& o, double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp_in_range(double x) {
-  const double y = rcp_seed(x);
-  const double e = fma(-x, y, 1.0);
+  const double e = fma(-x, y, o.one);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double rcp_any(double x) {
+__device__ __forceinline__ double rcp_any(const Ops& o, double x) {
   const int eb = (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
   if (eb < 1 || eb > 2044) return 1.0 / x;
-  return rcp_in_range(x);
+  return rcp_in_range(o, x);
 }
 
 // beta_0 of Eq. 2.20 from the scaled coefficients c[1..14]
-__device__ __forceinline__ double beta0(const double (&c)[15]) {
+__device__ __forceinline__ double beta0(const Ops& o, const double (&c)[15]) {
   // odd in one coordinate: (c1 + c6/4 + c8/12)^2 + 781/20 c6^2 + 47/10 c8^2, and c2, c9, c7
-  const double ta = fma(S1 / (12.0 * S3), c[8], fma(S1 / (4.0 * S3), c[6], c[1]));
-  const double tb = fma(S1 / (12.0 * S3), c[7], fma(S1 / (4.0 * S3), c[9], c[2]));
-  double b = (1.0 / S2) * fma(tb, tb, ta * ta);
-  b = fma(781.0 / (20.0 * S3 * S3), fma(c[9], c[9], c[6] * c[6]), b);
-  b = fma(47.0 / (10.0 * S3 * S3), fma(c[7], c[7], c[8] * c[8]), b);
+  const double k8 = K(B_A8), k6 = K(B_A6);
+  const double ta = fma(k8, c[8], fma(k6, c[6], c[1]));
+  const double tb = fma(k8, c[7], fma(k6, c[9], c[2]));
+  double b = o.mul(K(B_W1), fma(tb, tb, o.mul(ta, ta)));
+  b = fma(K(B_W6), fma(c[9], c[9], o.mul(c[6], c[6])), b);
+  b = fma(K(B_W8), fma(c[7], c[7], o.mul(c[8], c[8])), b);
   // even in both: 13/3 (c3 + 63/130 c10 + c12/12)^2 + 1421461/2275 c10^2, c5, c14, and c12^2
-  const double c12 = (S2 / (12.0 * S4)) * c[12];
-  const double tc = fma(63.0 * S2 / (130.0 * S4), c[10], c[3] + c12);
-  const double td = fma(63.0 * S2 / (130.0 * S4), c[14], c[5] + c12);
-  b = fma(13.0 / (3.0 * S2 * S2), fma(td, td, tc * tc), b);
-  b = fma(1421461.0 / (2275.0 * S4 * S4), fma(c[14], c[14], c[10] * c[10]), b);
-  b = fma(5083.0 * 144.0 / (270.0 * S2 * S2) * c12, c12, b);
+  const double c12 = o.mul(K(B_C12), c[12]), k10 = K(B_C10);
+  const double tc = fma(k10, c[10], o.add(c[3], c12));
+  const double td = fma(k10, c[14], o.add(c[5], c12));
+  b = fma(K(B_W3), fma(td, td, o.mul(tc, tc)), b);
+  b = fma(K(B_W10), fma(c[14], c[14], o.mul(c[10], c[10])), b);
+  b = fma(o.mul(K(B_W12), c12), c12, b);
   // odd in both: 7/6 (c4 + 17/70 (c11 + c13))^2 + 42.3.. (c11^2 + c13^2) - c11 c13 / 8400
-  const double p = c[11] + c[13], m = c[11] - c[13];
-  const double te = fma(17.0 * S2 / (70.0 * S4), p, c[4]);
-  b = fma(7.0 / (6.0 * S2 * S2) * te, te, b);
-  b = fma(710728.0 / (33600.0 * S4 * S4) * p, p, b);
-  b = fma(710730.0 / (33600.0 * S4 * S4) * m, m, b);
+  const double p = o.add(c[11], c[13]), m = o.sub(c[11], c[13]);
+  const double te = fma(K(B_E), p, c[4]);
+  b = fma(o.mul(K(B_W4), te), te, b);
+  b = fma(o.mul(K(B_WP), p), p, b);
+  b = fma(o.mul(K(B_WM), m), m, b);
   return b;
 }
 
@@ -84,37 +169,42 @@ struct Factors {
 // nonlinear_weights_fast, in the sums the combination needs and with d_m scaled by 25 (the
 // squared divisor of u_ave); the direct formula where the products leave the double range.
 template <bool ZERO_MEAN>
-__device__ __forceinline__ bool factors(double bt0, const double (&e)[4], double w5,
+__device__ __forceinline__ bool factors(const Ops& o, double bt0, const double (&e)[4], double w5,
                                         const KProblem& P, Factors& F) {
-  const double el2 = e[0] * e[0], er2 = e[1] * e[1], eb2 = e[2] * e[2], et2 = e[3] * e[3];
-  const double b1 = el2 + eb2, b2 = er2 + eb2, b3 = el2 + et2, b4 = er2 + et2;
-  const double s = (fabs(bt0 - b1) + fabs(bt0 - b2)) + (fabs(bt0 - b3) + fabs(bt0 - b4));
-  const double tau = (25.0 / 16.0) * s * s;  // 25 tau
+  const double el2 = o.mul(e[0], e[0]), er2 = o.mul(e[1], e[1]), eb2 = o.mul(e[2], e[2]),
+               et2 = o.mul(e[3], e[3]);
+  const double b1 = o.add(el2, eb2), b2 = o.add(er2, eb2), b3 = o.add(el2, et2),
+               b4 = o.add(er2, et2);
+  const double s = o.add(o.add(fabs(o.sub(bt0, b1)), fabs(o.sub(bt0, b2))),
+                         o.add(fabs(o.sub(bt0, b3)), fabs(o.sub(bt0, b4))));
+  const double tau = o.mul(o.mul(K(W_TAU), s), s);  // 25 tau
   double a;
   if constexpr (ZERO_MEAN)
-    a = (fabs(e[0]) + fabs(e[1])) + (fabs(e[2]) + fabs(e[3]));
+    a = o.add(o.add(fabs(e[0]), fabs(e[1])), o.add(fabs(e[2]), fabs(e[3])));
   else
-    a = (fabs(w5 - e[0]) + fabs(w5 + e[1])) + (fabs(w5 - e[2]) + fabs(w5 + e[3])) + fabs(w5);
-  const double ua = P.wmode == 1 ? 25.0 : a * a;  // 25 u_ave
-  const double eps = 25.0 * P.eps;
+    a = o.add(o.add(o.add(fabs(o.sub(w5, e[0])), fabs(o.add(w5, e[1]))),
+                    o.add(fabs(o.sub(w5, e[2])), fabs(o.add(w5, e[3])))), fabs(w5));
+  double ua = o.mul(a, a);  // 25 u_ave
+  if (P.wmode == 1) ua = 25.0;
+  const double eps = K(EPS);
   const double d0 = fma(bt0, ua, eps), d1 = fma(b1, ua, eps), d2 = fma(b2, ua, eps),
                d3 = fma(b3, ua, eps), d4 = fma(b4, ua, eps);
-  const double p12 = d1 * d2, p34 = d3 * d4;
-  const double D0 = p12 * p34, D = D0 * d0;
-  const double A = d0 * p34, B = d0 * p12;  // D1 = A d2, D2 = A d1, D3 = B d4, D4 = B d3
-  const double q12 = A * (d1 + d2), q34 = B * (d3 + d4);
-  const double q13 = fma(A, d2, B * d4);
-  const double q = q12 + q34, q24 = q - q13;
+  const double p12 = o.mul(d1, d2), p34 = o.mul(d3, d4);
+  const double D0 = o.mul(p12, p34), D = o.mul(D0, d0);
+  const double A = o.mul(d0, p34), B = o.mul(d0, p12);  // D1 = A d2, D2 = A d1, D3 = B d4, D4 = B d3
+  const double q12 = o.mul(A, o.add(d1, d2)), q34 = o.mul(B, o.add(d3, d4));
+  const double q13 = fma(A, d2, o.mul(B, d4));
+  const double q = o.add(q12, q34), q24 = o.sub(q, q13);
   const double N0 = fma(tau, D0, D);
-  const double S = fma(tau, fma(P.glo, q, P.g0[1] * D0), D);
+  const double S = fma(tau, fma(K(GLO), q, o.mul(K(G0), D0)), D);
   const long long eD = (__double_as_longlong(D) >> 52) & 0x7ff;
   const long long eS = (__double_as_longlong(S) >> 52) & 0x7ff;
   const bool ok = eD > 64 && eD < 2047 - 64 && eS > 64 && eS < 2047 - 64;
   const bool lin = P.wmode == 2;
-  const double inv = rcp_in_range(S);
-  const double k = (S1 * P.glo) * (tau * inv);
-  const double k0 = -2.0 * (k * D0);
-  F.a0 = lin ? 1.0 : N0 * inv;
+  const double inv = rcp_in_range(o, S);
+  const double k = o.mul(K(SGLO), o.mul(tau, inv));
+  const double k0 = o.mul(K(MTWO), o.mul(k, D0));
+  F.a0 = lin ? 1.0 : o.mul(N0, inv);
   F.l = lin ? 0.0 : fma(k, q13, k0);
   F.r = lin ? 0.0 : fma(k, q24, k0);
   F.b = lin ? 0.0 : fma(k, q12, k0);
@@ -140,53 +230,53 @@ __device__ __forceinline__ constexpr int role(int n) {
 }
 
 // the constant term of the polynomial with cell average `mean`
-__device__ __forceinline__ double constant_term(const double (&C)[15], double mean) {
-  return fma(-25.0 / 81.0, C[12], fma(-5.0 / 9.0, (C[3] + C[10]) + (C[5] + C[14]), mean));
+__device__ __forceinline__ double constant_term(const Ops& o, const double (&C)[15], double mean) {
+  return fma(K(M12), C[12], fma(K(MX), o.add(o.add(C[3], C[10]), o.add(C[5], C[14])), mean));
 }
 // the first-moment modification of direction DIR
 template <int DIR>
-__device__ __forceinline__ double vhat(const double (&C)[15]) {
-  return fma(1.0 / (144.0 * S3), C[role<DIR>(8)],
-             fma(1.0 / (80.0 * S3), C[role<DIR>(6)], (1.0 / (12.0 * S1)) * C[role<DIR>(1)]));
+__device__ __forceinline__ double vhat(const Ops& o, const double (&C)[15]) {
+  return fma(K(V8), C[role<DIR>(8)], fma(K(V6), C[role<DIR>(6)], o.mul(K(V1), C[role<DIR>(1)])));
 }
 // values on the two edges normal to direction DIR, at the three Gauss points along them
 // (C[0] set): lo = {(-1/2, -s), (-1/2, 0), (-1/2, s)}, hi the same at +1/2
 template <int DIR>
-__device__ __forceinline__ void edges(const double (&C)[15], double (&lo)[3], double (&hi)[3]) {
-  constexpr double h = 0.5 / S1, h2 = 0.25 / S2, h3 = 0.125 / S3, h4 = 0.0625 / S4;
+__device__ __forceinline__ void edges(const Ops& o, const double (&C)[15], double (&lo)[3],
+                                      double (&hi)[3]) {
 #define CC(n) C[role<DIR>(n)]
-  const double E0 = fma(h4, CC(10), fma(h2, CC(3), C[0]));
-  const double O0 = fma(h3, CC(6), h * CC(1));
-  const double Ev = E0 + fma(h2, CC(12), CC(5) + CC(14));
+  const double h = K(H1), h2 = K(H2), h3 = K(H3);
+  const double E0 = fma(K(H4), CC(10), fma(h2, CC(3), C[0]));
+  const double O0 = fma(h3, CC(6), o.mul(h, CC(1)));
+  const double Ev = o.add(E0, fma(h2, CC(12), o.add(CC(5), CC(14))));
   const double Od = fma(h, CC(8), O0);
-  const double Eo = fma(h2, CC(7), CC(2)) + CC(9);
-  const double Oo = fma(h3, CC(11), h * (CC(4) + CC(13)));
+  const double Eo = o.add(fma(h2, CC(7), CC(2)), CC(9));
+  const double Oo = fma(h3, CC(11), o.mul(h, o.add(CC(4), CC(13))));
 #undef CC
-  const double Pp = Ev + Oo, Pm = Ev - Oo, Qp = Od + Eo, Qm = Od - Eo;
-  hi[2] = Pp + Qp;   // (+, +): even + odd-even + even-odd + odd-odd
-  lo[0] = Pp - Qp;   // (-, -)
-  hi[0] = Pm + Qm;   // (+, -)
-  lo[2] = Pm - Qm;   // (-, +)
-  hi[1] = E0 + O0;
-  lo[1] = E0 - O0;
+  const double Pp = o.add(Ev, Oo), Pm = o.sub(Ev, Oo), Qp = o.add(Od, Eo), Qm = o.sub(Od, Eo);
+  hi[2] = o.add(Pp, Qp);   // (+, +): even + odd-even + even-odd + odd-odd
+  lo[0] = o.sub(Pp, Qp);   // (-, -)
+  hi[0] = o.add(Pm, Qm);   // (+, -)
+  lo[2] = o.sub(Pm, Qm);   // (-, +)
+  hi[1] = o.add(E0, O0);
+  lo[1] = o.sub(E0, O0);
 }
 // values at the nine interior Gauss points, index 3 (1 + xi/s) + (1 + eta/s)
-__device__ __forceinline__ void interior(const double (&C)[15], double (&in)[9]) {
-  const double ex = C[3] + C[10], ey = C[5] + C[14];
-  const double EX = C[0] + ex, EY = C[0] + ey;
-  const double EE = (EX + ey) + C[12];
-  const double ox = C[1] + C[6], oy = C[2] + C[9];
-  const double OE = ox + C[8], EO = oy + C[7];
-  const double OO = C[4] + (C[11] + C[13]);
-  const double Pp = EE + OO, Pm = EE - OO, Qp = OE + EO, Qm = OE - EO;
-  in[8] = Pp + Qp;
-  in[0] = Pp - Qp;
-  in[6] = Pm + Qm;
-  in[2] = Pm - Qm;
-  in[7] = EX + ox;
-  in[1] = EX - ox;
-  in[5] = EY + oy;
-  in[3] = EY - oy;
+__device__ __forceinline__ void interior(const Ops& o, const double (&C)[15], double (&in)[9]) {
+  const double ex = o.add(C[3], C[10]), ey = o.add(C[5], C[14]);
+  const double EX = o.add(C[0], ex), EY = o.add(C[0], ey);
+  const double EE = o.add(o.add(EX, ey), C[12]);
+  const double ox = o.add(C[1], C[6]), oy = o.add(C[2], C[9]);
+  const double OE = o.add(ox, C[8]), EO = o.add(oy, C[7]);
+  const double OO = o.add(C[4], o.add(C[11], C[13]));
+  const double Pp = o.add(EE, OO), Pm = o.sub(EE, OO), Qp = o.add(OE, EO), Qm = o.sub(OE, EO);
+  in[8] = o.add(Pp, Qp);
+  in[0] = o.sub(Pp, Qp);
+  in[6] = o.add(Pm, Qm);
+  in[2] = o.sub(Pm, Qm);
+  in[7] = o.add(EX, ox);
+  in[1] = o.sub(EX, ox);
+  in[5] = o.add(EY, oy);
+  in[3] = o.sub(EY, oy);
   in[4] = C[0];
 }
 
@@ -196,10 +286,10 @@ __device__ __forceinline__ void interior(const double (&C)[15], double (&in)[9])
 // row window adds): the window [3 rows][12][BW + 2]; the x-face exchange [12][BW] (f - a1 u of
 // each cell's left trace, then the Gauss moments of the face's flux); g + a2 u of the top
 // traces carried to the next row [12][BW]; the coefficients of X/2, q_x, q_y [42][BW]; the
-// entropy field's point values and modifications [23][BW].
+// entropy field's point values and modifications [23][BW]; and the table of constants.
 template <int BW>
 constexpr size_t smem_bytes_char64() {
-  return sizeof(double) * (36 * (BW + 2) + (12 + 12 + 42 + 23) * BW);
+  return sizeof(double) * (36 * (BW + 2) + (12 + 12 + 42 + 23) * BW + c64::kTable);
 }
 
 template <int BW>
@@ -214,6 +304,8 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
   double* car = xch + 12 * BW + t;       // this thread's column
   double* cf = xch + 24 * BW + t;        // this thread's column: X/2 (0-13), q_x, q_y
   double* w1p = cf + 42 * BW;            // this thread's column: W1 on x edges, y edges, inside
+  double* tab = xch + (24 + 42 + 23) * BW;
+  fill_table(tab, P);
   const int nx = P.nx, ny = P.ny;
   const size_t plane = (size_t)nx * ny;
   const int i0 = band * wout;
@@ -250,6 +342,10 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
 #pragma unroll 1
   for (int r = j0 - 2; r <= j0; ++r) load_row(r);
   __syncthreads();
+  Ops o;
+  o.tab = (unsigned)__cvta_generic_to_shared(tab) + (unsigned)((S.k >> 2) * t);  // k <= 3: + 0
+  o.one = K(ONE);
+  o.nz = K(NZERO);
 
   double pend[NC][3];              // F^1..F^3 of (i, j-1) without its top face
   double pvh[NC], pwh[NC];         // v-hat, w-hat of (i, j-1)
@@ -273,58 +369,60 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
       {
         const double U0 = w0[0 * WC + t + 1], U1 = w0[3 * WC + t + 1], U2 = w0[6 * WC + t + 1],
                      U3 = w0[9 * WC + t + 1];
-        const double ir = rcp_any(U0);
-        vx = U1 * ir;
-        vy = U2 * ir;
-        q2h = 0.5 * fma(vx, vx, vy * vy);
-        p5 = P.gm1 * fma(-U0, q2h, U3);
-        c2 = P.gam * p5 * ir;
+        const double ir = rcp_any(o, U0);
+        vx = o.mul(U1, ir);
+        vy = o.mul(U2, ir);
+        q2h = o.mul(K(HALF), fma(vx, vx, o.mul(vy, vy)));
+        p5 = o.mul(K(GM1), fma(-U0, q2h, U3));
+        c2 = o.mul(o.mul(K(GAM), p5), ir);
         const double rc = rsqrt(c2);
-        c = c2 * rc;
-        h = fma(U3 + p5, ir, -q2h);
-        hic = 0.5 * rc;
-        const double rc2 = rc * rc;
-        b1h = 0.5 * P.gm1 * rc2;
-        X5 = p5 * rc2;
+        c = o.mul(c2, rc);
+        h = fma(o.add(U3, p5), ir, -q2h);
+        hic = o.mul(K(HALF), rc);
+        const double rc2 = o.mul(rc, rc);
+        b1h = -o.mul(K(HGM1), rc2);
+        X5 = o.mul(p5, rc2);
       }
       // the 14 stencil combinations of the conserved components
       //  0 X1, 1 Va, 2 X2, 3 Wa, 4 X3, 5 v82, 6 w64, 7 corners - 4 u5, 8 Vd, 9 Wd,
       //  10 u5 - u4, 11 u6 - u5, 12 u5 - u2, 13 u8 - u5
 #pragma unroll
       for (int a = 0; a < NC; ++a) {
-        double* o = a == 0 ? w1p : cf + (a == 3 ? 0 : 14 * a) * BW;
+        double* s = a == 0 ? w1p : cf + (a == 3 ? 0 : 14 * a) * BW;
         const double* m0 = wm + 3 * a * WC + t;
         const double* m1 = w0 + 3 * a * WC + t;
         const double* m2 = wp + 3 * a * WC + t;
         const double u1 = m0[0], u3 = m0[2], u7 = m2[0], u9 = m2[2];
-        const double sb = u1 + u3, st = u7 + u9, db = u1 - u3, dtp = u7 - u9;
-        o[0 * BW] = db + dtp;
-        o[2 * BW] = sb - st;
-        o[4 * BW] = db - dtp;
+        const double sb = o.add(u1, u3), st = o.add(u7, u9), db = o.sub(u1, u3),
+                     dtp = o.sub(u7, u9);
+        s[0 * BW] = o.add(db, dtp);
+        s[2 * BW] = o.sub(sb, st);
+        s[4 * BW] = o.sub(db, dtp);
         const double u5 = m1[1];
-        o[7 * BW] = fma(-4.0, u5, sb + st);
-        o[10 * BW] = u5 - m1[0];
-        o[11 * BW] = m1[2] - u5;
-        o[12 * BW] = u5 - m0[1];
-        o[13 * BW] = m2[1] - u5;
+        s[7 * BW] = fma(K(MFOUR), u5, o.add(sb, st));
+        s[10 * BW] = o.sub(u5, m1[0]);
+        s[11 * BW] = o.sub(m1[2], u5);
+        s[12 * BW] = o.sub(u5, m0[1]);
+        s[13 * BW] = o.sub(m2[1], u5);
         const double v4 = m1[WC], v6 = m1[WC + 2];
-        o[1 * BW] = v4 + v6;
-        o[8 * BW] = v6 - v4;
-        o[5 * BW] = m2[WC + 1] - m0[WC + 1];
+        s[1 * BW] = o.add(v4, v6);
+        s[8 * BW] = o.sub(v6, v4);
+        s[5 * BW] = o.sub(m2[WC + 1], m0[WC + 1]);
         const double z2 = m0[2 * WC + 1], z8 = m2[2 * WC + 1];
-        o[3 * BW] = z2 + z8;
-        o[9 * BW] = z8 - z2;
-        o[6 * BW] = m1[2 * WC + 2] - m1[2 * WC];
+        s[3 * BW] = o.add(z2, z8);
+        s[9 * BW] = o.sub(z8, z2);
+        s[6 * BW] = o.sub(m1[2 * WC + 2], m1[2 * WC]);
       }
       // into the frame, in place: (rho, m_x, m_y, E) -> (W1, q_x, q_y, X/2)
       double dW[4];
-      const double bx = b1h * vx, by = b1h * vy, bq = b1h * q2h;
+      const double bx = o.mul(b1h, vx), by = o.mul(b1h, vy), bq = o.mul(b1h, q2h);
+      const double m2 = K(MTWO);
 #pragma unroll
       for (int n = 0; n < 14; ++n) {
         const double r = w1p[n * BW];
         const double qx = fma(-vx, r, cf[(14 + n) * BW]), qy = fma(-vy, r, cf[(28 + n) * BW]);
-        const double xh = fma(-bq, r, fma(-by, qy, fma(-bx, qx, b1h * cf[n * BW])));
-        const double w1 = fma(-2.0, xh, r);
+        const double xh = fma(-bq, r, fma(-by, qy, fma(-bx, qx, o.mul(b1h, cf[n * BW]))));
+        const double w1 = fma(m2, xh, r);
         if (n >= 10) {
           dX[n - 10] = xh;
           dqx[n - 10] = qx;
@@ -338,80 +436,83 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
         }
       }
       // the Appendix coefficients (scaled) of one variable from its combinations
-      auto coefficients = [&](const double* o, const double (&e)[4], double (&C)[15]) {
+      auto coefficients = [&](const double* s, const double (&e)[4], double (&C)[15]) {
         {
-          const double X1 = o[0 * BW], Va = o[1 * BW], ee = -(e[0] + e[1]);
-          C[1] = fma(-75.0 / 19.0 * S1, Va, fma(-397.0 / 456.0 * S1, ee, S1 / 48.0 * X1));
-          C[6] = fma(60.0 / 19.0 * S3, Va, 5.0 / 19.0 * S3 * ee);
-          C[8] = fma(0.5 * S3, ee, -0.25 * S3 * X1);
+          const double X1 = s[0 * BW], Va = s[1 * BW], ex = -o.add(e[0], e[1]);
+          const double X2 = s[2 * BW], Wa = s[3 * BW], ey = -o.add(e[2], e[3]);
+          const double kx = K(A1X), ke = K(A1E), kv = K(A1V);
+          C[1] = fma(kv, Va, fma(ke, ex, o.mul(kx, X1)));
+          C[2] = fma(kv, Wa, fma(ke, ey, o.mul(kx, X2)));
+          const double k6 = K(A6E), k6v = K(A6V);
+          C[6] = fma(k6v, Va, o.mul(k6, ex));
+          C[9] = fma(k6v, Wa, o.mul(k6, ey));
+          const double k8 = K(A8X), k8e = K(A8E);
+          C[8] = fma(k8e, ex, o.mul(k8, X1));
+          C[7] = fma(k8e, ey, o.mul(k8, X2));
         }
         {
-          const double X2 = o[2 * BW], Wa = o[3 * BW], ee = -(e[2] + e[3]);
-          C[2] = fma(-75.0 / 19.0 * S1, Wa, fma(-397.0 / 456.0 * S1, ee, S1 / 48.0 * X2));
-          C[9] = fma(60.0 / 19.0 * S3, Wa, 5.0 / 19.0 * S3 * ee);
-          C[7] = fma(0.5 * S3, ee, -0.25 * S3 * X2);
+          const double X3 = s[4 * BW], v82 = s[5 * BW], w64 = s[6 * BW];
+          C[4] = fma(K(A4X), X3, o.mul(K(A4V), o.add(v82, w64)));
+          const double x = o.mul(K(A11X), X3), kv = K(A11V);
+          C[11] = fma(kv, v82, x);
+          C[13] = fma(kv, w64, x);
         }
         {
-          const double X3 = o[4 * BW], v82 = o[5 * BW], w64 = o[6 * BW];
-          C[4] = fma(-7.0 / 22.0 * S2, X3, 75.0 / 11.0 * S2 * (v82 + w64));
-          const double x = 5.0 / 22.0 * S4 * X3;
-          C[11] = fma(-60.0 / 11.0 * S4, v82, x);
-          C[13] = fma(-60.0 / 11.0 * S4, w64, x);
-        }
-        {
-          const double r = o[7 * BW], Vd = o[8 * BW], Wd = o[9 * BW];
-          const double p = e[1] - e[0], q = e[3] - e[2];
-          const double rr = -S2 / 48.0 * r;
-          C[3] = fma(-45.0 / 8.0 * S2, Vd, fma(71.0 / 48.0 * S2, p, fma(S2 / 24.0, q, rr)));
-          C[5] = fma(-45.0 / 8.0 * S2, Wd, fma(71.0 / 48.0 * S2, q, fma(S2 / 24.0, p, rr)));
-          C[10] = fma(15.0 / 4.0 * S4, Vd, -5.0 / 8.0 * S4 * p);
-          C[14] = fma(15.0 / 4.0 * S4, Wd, -5.0 / 8.0 * S4 * q);
-          C[12] = fma(-0.5 * S4, q, fma(-0.5 * S4, p, 0.25 * S4 * r));
+          const double r = s[7 * BW], Vd = s[8 * BW], Wd = s[9 * BW];
+          const double p = o.sub(e[1], e[0]), q = o.sub(e[3], e[2]);
+          const double rr = o.mul(K(A3R), r), kq = K(A3Q), kp = K(A3P), kv = K(A3V);
+          C[3] = fma(kv, Vd, fma(kp, p, fma(kq, q, rr)));
+          C[5] = fma(kv, Wd, fma(kp, q, fma(kq, p, rr)));
+          const double k10 = K(A10P), k10v = K(A10V);
+          C[10] = fma(k10v, Vd, o.mul(k10, p));
+          C[14] = fma(k10v, Wd, o.mul(k10, q));
+          const double k12 = K(A12P);
+          C[12] = fma(k12, q, fma(k12, p, o.mul(K(A12R), r)));
         }
       };
       // X/2, q_x, q_y: their coefficients replace their combinations
 #pragma unroll 1
       for (int v = 0; v < 3; ++v) {
-        double* o = cf + 14 * v * BW;
+        double* s = cf + 14 * v * BW;
         double C[15], e[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n) e[n] = v == 0 ? dX[n] : (v == 1 ? dqx[n] : dqy[n]);
-        coefficients(o, e, C);
+        coefficients(s, e, C);
 #pragma unroll
-        for (int n = 0; n < 14; ++n) o[n * BW] = C[n + 1];
+        for (int n = 0; n < 14; ++n) s[n * BW] = C[n + 1];
       }
       // the entropy field: reconstructed here for both passes
       {
         double C[15];
         coefficients(w1p, dW, C);
         Factors F;
-        const double mean = w0[0 * WC + t + 1] - X5;
-        fast &= factors<false>(beta0(C), dW, mean, P, F);
+        const double mean = o.sub(w0[0 * WC + t + 1], X5);
+        fast &= factors<false>(o, beta0(o, C), dW, mean, P, F);
 #pragma unroll
-        for (int n = 1; n < 15; ++n) C[n] *= F.a0;
+        for (int n = 1; n < 15; ++n) C[n] = o.mul(C[n], F.a0);
         C[1] = fma(F.r, dW[1], fma(F.l, dW[0], C[1]));
         C[2] = fma(F.t, dW[3], fma(F.b, dW[2], C[2]));
-        C[0] = constant_term(C, mean);
+        C[0] = constant_term(o, C, mean);
         double lo[3], hi[3];
-        edges<1>(C, lo, hi);
+        edges<1>(o, C, lo, hi);
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
           w1p[(6 + g) * BW] = lo[g];
           w1p[(9 + g) * BW] = hi[g];
         }
         if (xrow) {
-          edges<0>(C, lo, hi);
+          edges<0>(o, C, lo, hi);
 #pragma unroll
           for (int g = 0; g < 3; ++g) {
             w1p[g * BW] = lo[g];
             w1p[(3 + g) * BW] = hi[g];
           }
           double in[9];
-          interior(C, in);
+          interior(o, C, in);
 #pragma unroll
           for (int g = 0; g < 9; ++g) w1p[(12 + g) * BW] = in[g];
-          w1p[21 * BW] = vhat<0>(C);
-          w1p[22 * BW] = vhat<1>(C);
+          w1p[21 * BW] = vhat<0>(o, C);
+          w1p[22 * BW] = vhat<1>(o, C);
         }
       }
     }
@@ -440,6 +541,7 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
         // the acoustic fields X/2 -+ q_n/(2c), then X = W0 + W3 and q_n = c (W3 - W0)
         {
           Factors F0, F3;
+          const double w5 = o.mul(K(HALF), X5);
           double s0x, s0y, s3x, s3y;
           {
             double C[15], e[4];
@@ -447,9 +549,9 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
             for (int n = 1; n < 15; ++n) C[n] = fma(-hic, cN[(n - 1) * BW], cX[(n - 1) * BW]);
 #pragma unroll
             for (int n = 0; n < 4; ++n) e[n] = fma(-hic, eN[n], dX[n]);
-            fast &= factors<false>(beta0(C), e, 0.5 * X5, P, F0);
-            s0x = fma(F0.r, e[1], F0.l * e[0]);
-            s0y = fma(F0.t, e[3], F0.b * e[2]);
+            fast &= factors<false>(o, beta0(o, C), e, w5, P, F0);
+            s0x = fma(F0.r, e[1], o.mul(F0.l, e[0]));
+            s0y = fma(F0.t, e[3], o.mul(F0.b, e[2]));
           }
           {
             double C[15], e[4];
@@ -457,118 +559,118 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
             for (int n = 1; n < 15; ++n) C[n] = fma(hic, cN[(n - 1) * BW], cX[(n - 1) * BW]);
 #pragma unroll
             for (int n = 0; n < 4; ++n) e[n] = fma(hic, eN[n], dX[n]);
-            fast &= factors<false>(beta0(C), e, 0.5 * X5, P, F3);
-            s3x = fma(F3.r, e[1], F3.l * e[0]);
-            s3y = fma(F3.t, e[3], F3.b * e[2]);
+            fast &= factors<false>(o, beta0(o, C), e, w5, P, F3);
+            s3x = fma(F3.r, e[1], o.mul(F3.l, e[0]));
+            s3y = fma(F3.t, e[3], o.mul(F3.b, e[2]));
           }
-          const double ap = F0.a0 + F3.a0, am = F3.a0 - F0.a0;
-          const double xq = hic * am, qx = c * am, qq = 0.5 * ap;
+          const double ap = o.add(F0.a0, F3.a0), am = o.sub(F3.a0, F0.a0);
+          const double xq = o.mul(hic, am), qx = o.mul(c, am), qq = o.mul(K(HALF), ap);
 #pragma unroll
           for (int n = 1; n < 15; ++n) {
             const double x = cX[(n - 1) * BW], q = cN[(n - 1) * BW];
-            PX[n] = fma(xq, q, ap * x);
-            PQ[n] = fma(qq, q, qx * x);
+            PX[n] = fma(xq, q, o.mul(ap, x));
+            PQ[n] = fma(qq, q, o.mul(qx, x));
           }
-          PX[1] += s0x + s3x;
-          PX[2] += s0y + s3y;
-          PQ[1] = fma(c, s3x - s0x, PQ[1]);
-          PQ[2] = fma(c, s3y - s0y, PQ[2]);
-          PX[0] = constant_term(PX, X5);
-          PQ[0] = constant_term(PQ, 0.0);
+          PX[1] = o.add(PX[1], o.add(s0x, s3x));
+          PX[2] = o.add(PX[2], o.add(s0y, s3y));
+          PQ[1] = fma(c, o.sub(s3x, s0x), PQ[1]);
+          PQ[2] = fma(c, o.sub(s3y, s0y), PQ[2]);
+          PX[0] = constant_term(o, PX, X5);
+          PQ[0] = constant_term(o, PQ, o.nz);
         }
         // the shear field: the tangential momentum in the cell's frame
         {
 #pragma unroll
           for (int n = 1; n < 15; ++n) PT[n] = cT[(n - 1) * BW];
           Factors F;
-          fast &= factors<true>(beta0(PT), eT, 0.0, P, F);
+          fast &= factors<true>(o, beta0(o, PT), eT, 0.0, P, F);
 #pragma unroll
-          for (int n = 1; n < 15; ++n) PT[n] *= F.a0;
+          for (int n = 1; n < 15; ++n) PT[n] = o.mul(PT[n], F.a0);
           PT[1] = fma(F.r, eT[1], fma(F.l, eT[0], PT[1]));
           PT[2] = fma(F.t, eT[3], fma(F.b, eT[2], PT[2]));
-          PT[0] = constant_term(PT, 0.0);
+          PT[0] = constant_term(o, PT, o.nz);
         }
         // conserved components of the frame variables (rho, q_n, q_t, X)
         auto conserved = [&](double r, double q, double s, double x, double& mn, double& mt,
                              double& E) {
           mn = fma(un, r, q);
           mt = fma(ut, r, s);
-          E = fma(q2h, r, fma(ut, s, fma(un, q, h * x)));
+          E = fma(q2h, r, fma(ut, s, fma(un, q, o.mul(h, x))));
         };
         // traces and their fluxes
         {
           double X[2][3], Q[2][3], T[2][3];
           if (dir == 0) {
-            edges<0>(PX, X[0], X[1]);
-            edges<0>(PQ, Q[0], Q[1]);
-            edges<0>(PT, T[0], T[1]);
+            edges<0>(o, PX, X[0], X[1]);
+            edges<0>(o, PQ, Q[0], Q[1]);
+            edges<0>(o, PT, T[0], T[1]);
           } else {
-            edges<1>(PX, X[0], X[1]);
-            edges<1>(PQ, Q[0], Q[1]);
-            edges<1>(PT, T[0], T[1]);
+            edges<1>(o, PX, X[0], X[1]);
+            edges<1>(o, PQ, Q[0], Q[1]);
+            edges<1>(o, PT, T[0], T[1]);
           }
-          const double a = dir == 0 ? a1 : a2;
+          const double a = dir == 0 ? a1 : a2, gm1 = K(GM1), hg = K(HGM1);
 #pragma unroll
           for (int side = 0; side < 2; ++side)
 #pragma unroll
             for (int g = 0; g < 3; ++g) {
-              const double r = w1p[(6 * dir + 3 * side + g) * BW] + X[side][g];
+              const double r = o.add(w1p[(6 * dir + 3 * side + g) * BW], X[side][g]);
               double mn, mt, E;
               conserved(r, Q[side][g], T[side][g], X[side][g], mn, mt, E);
-              const double ir = rcp_any(r);
-              const double vn = mn * ir;
-              const double kin = fma(mn, mn, mt * mt) * ir;
-              const double p = fma(-0.5 * P.gm1, kin, P.gm1 * E);
-              const double fn = fma(mn, vn, p), ft = mt * vn, fE = (E + p) * vn;
-              double(&o)[NC] = side == 0 ? glo[g] : ghi[g];
+              const double ir = rcp_any(o, r);
+              const double vn = o.mul(mn, ir);
+              const double kin = o.mul(fma(mn, mn, o.mul(mt, mt)), ir);
+              const double p = fma(hg, kin, o.mul(gm1, E));
+              const double fn = fma(mn, vn, p), ft = o.mul(mt, vn), fE = o.mul(o.add(E, p), vn);
+              double(&f)[NC] = side == 0 ? glo[g] : ghi[g];
               const double as = side == 0 ? -a : a;
-              o[0] = fma(as, r, mn);
-              o[dir == 0 ? 1 : 2] = fma(as, mn, fn);
-              o[dir == 0 ? 2 : 1] = fma(as, mt, ft);
-              o[3] = fma(as, E, fE);
+              f[0] = fma(as, r, mn);
+              f[dir == 0 ? 1 : 2] = fma(as, mn, fn);
+              f[dir == 0 ? 2 : 1] = fma(as, mt, ft);
+              f[3] = fma(as, E, fE);
             }
         }
         // volume sum and first-moment modification
         if (xrow) {
           double X[9], Q[9], T[9];
-          interior(PX, X);
-          interior(PQ, Q);
-          interior(PT, T);
-          double K = 0.0, A = 0.0, B = 0.0, G1 = 0.0, G2 = 0.0;
+          interior(o, PX, X);
+          interior(o, PQ, Q);
+          interior(o, PT, T);
+          double Z = o.nz, A = o.nz, B = o.nz, G1 = o.nz, G2 = o.nz;
+          const double wc = K(WC), we = K(WE), wm_ = K(WM);
 #pragma unroll
           for (int g = 0; g < 9; ++g) {
-            const double r = w1p[(12 + g) * BW] + X[g];
-            const double w = g == 4 ? 16.0 / 81.0 : ((g & 1) ? 10.0 / 81.0 : 25.0 / 324.0);
-            const double ir = rcp_any(r);
-            const double wir = w * ir;
-            const double qa = Q[g] * wir;
-            const double z = fma(Q[g], Q[g], T[g] * T[g]);
-            K = fma(wir, z, K);
+            const double r = o.add(w1p[(12 + g) * BW], X[g]);
+            const double ir = rcp_any(o, r);
+            const double wir = o.mul(g == 4 ? wm_ : ((g & 1) ? we : wc), ir);
+            const double qa = o.mul(Q[g], wir);
+            const double z = fma(Q[g], Q[g], o.mul(T[g], T[g]));
+            Z = fma(wir, z, Z);
             A = fma(Q[g], qa, A);
             B = fma(T[g], qa, B);
             G1 = fma(X[g], qa, G1);
-            G2 = fma(qa * ir, z, G2);
+            G2 = fma(o.mul(qa, ir), z, G2);
           }
-          const double hg = 0.5 * P.gm1;
-          const double pm = fma(-hg, K, p5);
+          const double hg = K(HGM1);
+          const double pm = fma(hg, Z, p5);
           const double mn = w0[(dir == 0 ? 3 : 6) * WC + t + 1];
           const double mt = w0[(dir == 0 ? 6 : 3) * WC + t + 1];
           const double E = w0[9 * WC + t + 1];
           vol[0] = mn;
-          vol[dir == 0 ? 1 : 2] = fma(mn, un, A + pm);
+          vol[dir == 0 ? 1 : 2] = fma(mn, un, o.add(A, pm));
           vol[dir == 0 ? 2 : 1] = fma(mt, un, B);
-          vol[3] = fma(un, E + pm, fma(ut, B, fma(un, A, fma(h + c2, G1, -hg * G2))));
-          const double Xv = dir == 0 ? vhat<0>(PX) : vhat<1>(PX);
-          const double Qv = dir == 0 ? vhat<0>(PQ) : vhat<1>(PQ);
-          const double Tv = dir == 0 ? vhat<0>(PT) : vhat<1>(PT);
-          mod[0] = w1p[(21 + dir) * BW] + Xv;
+          vol[3] = fma(un, o.add(E, pm),
+                       fma(ut, B, fma(un, A, fma(o.add(h, c2), G1, o.mul(hg, G2)))));
+          const double Xv = dir == 0 ? vhat<0>(o, PX) : vhat<1>(o, PX);
+          const double Qv = dir == 0 ? vhat<0>(o, PQ) : vhat<1>(o, PQ);
+          const double Tv = dir == 0 ? vhat<0>(o, PT) : vhat<1>(o, PT);
+          mod[0] = o.add(w1p[(21 + dir) * BW], Xv);
           conserved(mod[0], Qv, Tv, Xv, mod[dir == 0 ? 1 : 2], mod[dir == 0 ? 2 : 1], mod[3]);
         }
       }
       if (dir == 0) {
         // x faces: twice the LF flux of a face is (f + a u) of the left cell's trace plus
         // (f - a u) of the right cell's; each face formed once, by the thread left of it
-        const double idx = P.inv_dx;
         if (need) {
 #pragma unroll
           for (int g = 0; g < 3; ++g)
@@ -577,24 +679,26 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
         }
         __syncthreads();
         if (need && t <= wout && i < nx) {
-          const double k0 = 5.0 / 36.0 * idx, k1 = 2.0 / 9.0 * idx, k2 = 5.0 / 36.0 * S1 * idx;
+          const double k0 = K(FX0), k1 = K(FX1), k2 = K(FX2);
 #pragma unroll
           for (int a = 0; a < NC; ++a) {
             double* x = xch + a * 3 * BW + t + 1;
-            const double F0 = ghi[0][a] + x[0], F1 = ghi[1][a] + x[BW], F2 = ghi[2][a] + x[2 * BW];
-            x[0] = fma(k1, F1, k0 * (F0 + F2));  // this thread is the slots' only reader
-            x[BW] = k2 * (F2 - F0);
+            const double F0 = o.add(ghi[0][a], x[0]), F1 = o.add(ghi[1][a], x[BW]),
+                         F2 = o.add(ghi[2][a], x[2 * BW]);
+            x[0] = fma(k1, F1, o.mul(k0, o.add(F0, F2)));  // the slots' only reader
+            x[BW] = o.mul(k2, o.sub(F2, F0));
           }
         }
         __syncthreads();
         if (outc) {
+          const double idx = K(IDX), half = K(HALF);
 #pragma unroll
           for (int a = 0; a < NC; ++a) {
             const double* x = xch + a * 3 * BW + t;
             const double Lw = x[0], Rw = x[1];
-            rx[a][0] = Lw - Rw;
-            rx[a][1] = fma(vol[a], idx, -0.5 * (Lw + Rw));
-            rx[a][2] = x[BW] - x[BW + 1];
+            rx[a][0] = o.sub(Lw, Rw);
+            rx[a][1] = fma(vol[a], idx, -o.mul(half, o.add(Lw, Rw)));
+            rx[a][2] = o.sub(x[BW], x[BW + 1]);
           }
         }
         if (need) {
@@ -610,10 +714,11 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
             gt[g][a] = ghi[g][a];
           }
         if (xrow) {
+          const double idy = K(IDY);
 #pragma unroll
           for (int a = 0; a < NC; ++a) {
             wh[a] = mod[a];
-            rx[a][2] = fma(vol[a], P.inv_dy, rx[a][2]);
+            rx[a][2] = fma(vol[a], idy, rx[a][2]);
           }
         }
       }
@@ -621,20 +726,20 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
 
     // y face j-1/2 between (i, j-1) (its top traces' part carried) and (i, j): Eq. 2.16
     if (need && j > j0 - 1) {
-      const double idy = P.inv_dy;
-      const double k0 = 5.0 / 36.0 * idy, k1 = 2.0 / 9.0 * idy, k2 = 5.0 / 36.0 * S1 * idy;
+      const double k0 = K(FY0), k1 = K(FY1), k2 = K(FY2), half = K(HALF);
 #pragma unroll
       for (int a = 0; a < NC; ++a) {
-        const double G0 = car[(a * 3 + 0) * BW] + gb[0][a], G1 = car[(a * 3 + 1) * BW] + gb[1][a],
-                     G2 = car[(a * 3 + 2) * BW] + gb[2][a];
-        const double sw = fma(k1, G1, k0 * (G0 + G2));
-        const double sm = k2 * (G2 - G0);
-        pend[a][0] -= sw;
-        pend[a][1] -= sm;
-        pend[a][2] = fma(-0.5, sw, pend[a][2]);
-        rx[a][0] += sw;
-        rx[a][1] += sm;
-        rx[a][2] = fma(-0.5, sw, rx[a][2]);
+        const double G0 = o.add(car[(a * 3 + 0) * BW], gb[0][a]),
+                     G1 = o.add(car[(a * 3 + 1) * BW], gb[1][a]),
+                     G2 = o.add(car[(a * 3 + 2) * BW], gb[2][a]);
+        const double sw = fma(k1, G1, o.mul(k0, o.add(G0, G2)));
+        const double sm = o.mul(k2, o.sub(G2, G0));
+        pend[a][0] = o.sub(pend[a][0], sw);
+        pend[a][1] = o.sub(pend[a][1], sm);
+        pend[a][2] = fma(-half, sw, pend[a][2]);
+        rx[a][0] = o.add(rx[a][0], sw);
+        rx[a][1] = o.add(rx[a][1], sm);
+        rx[a][2] = fma(-half, sw, rx[a][2]);
       }
       // stage update of (i, j-1): Eq. 2.13
       if (outc && j - 1 >= j0) {
@@ -655,13 +760,13 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
               base = (m == 0) ? S.Un[qa] : S.Vh[(size_t)(a * 2 + m - 1) * plane + q];
             }
             const double adv = fma(dt, pend[a][m], own[m]);
-            double o;
-            if (S.k == 1) o = adv;
-            else if (S.k == 2) o = fma(0.75, base, 0.25 * adv);
-            else o = fma(1.0 / 3.0, base, 2.0 / 3.0 * adv);
-            S.Uout[qa] = o;
-            bad |= !finite_bits(o);
-            if (m == 0) ua[a] = o;
+            double out;
+            if (S.k == 1) out = adv;
+            else if (S.k == 2) out = fma(K(THREEQ), base, o.mul(K(QUARTER), adv));
+            else out = fma(K(THIRD), base, o.mul(K(TWOTHIRD), adv));
+            S.Uout[qa] = out;
+            bad |= !finite_bits(out);
+            if (m == 0) ua[a] = out;
           }
         }
         double s0, s1;
@@ -719,5 +824,7 @@ __device__ __forceinline__ void stage2d_char64_item(const KProblem& P, const KSt
   }
   __syncthreads();  // the block may start another item in the same shared memory
 }
+
+#undef K
 
 }  // namespace hw

@@ -1,22 +1,35 @@
 """The characteristic FP64 2D Euler stage at the edges of its bands and chunks, against the
 oracle: every stage, mixed boundary conditions, grids of one band and of ragged bands, through
 the single-solve and the batched launches.  Tolerance: the FP64 parity bar of the other stage
-tests (1e-12 of the component's scale per cell and moment)."""
+tests (1e-12 of the component's scale per cell and moment).  The states vary by a third about a
+mean, so that no reconstructed point comes near vacuum: there a flux m^2/rho amplifies rounding
+without bound, and the oracle itself is further than 1e-12 from the scheme evaluated in 80-bit
+arithmetic."""
 import numpy as np
 import pytest
 
 import oracle as O
 from paper_2402_03074_gb300 import _binding as H
-from paper_2402_03074_gb300 import inputs as I
 from gpu_helpers import gpu_stage, problems, rel_err
 
 pytestmark = pytest.mark.gpu
 
 
+def _state(nx, ny, seed):
+    rng = np.random.default_rng(seed)
+    U = np.zeros((4, 3, ny, nx))
+    U[0, 0] = rng.uniform(0.8, 1.2, (ny, nx))
+    U[1, 0] = rng.uniform(-0.6, 0.6, (ny, nx))
+    U[2, 0] = rng.uniform(-0.6, 0.6, (ny, nx))
+    U[3, 0] = rng.uniform(2.5, 3.0, (ny, nx))
+    U[:, 1:] = rng.uniform(-0.01, 0.01, (4, 2, ny, nx))
+    return U
+
+
 def _case(nx, ny, bc, k, weights):
     op, hp = problems(2, "euler", nx, ny, bc=bc, weights=weights)
-    U = I.random_state(op.shape, seed=nx * 7 + ny, eq=I.EULER)
-    Un = U if k == 1 else I.random_state(op.shape, seed=nx + ny, eq=I.EULER)
+    U = _state(nx, ny, nx * 7 + ny)
+    Un = U if k == 1 else _state(nx, ny, nx + ny)
     Vh = np.random.default_rng(nx).uniform(-0.05, 0.05, (4, 2, ny, nx))
     a = O.alpha(op, U)
     dt = 0.2 / 64.0 / a.sum()
