@@ -13,10 +13,13 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhweno.so")
-SOURCES = ["stage2d.cu", "stage2d_w96.cu", "stage2d_w64.cu", "stage2d_w192.cu", "stage1d.cu",
+SOURCES = ["stage2d.cu", "stage2d_w96.cu", "stage2d_w64.cu", "stage2d_w192.cu", "stage2d_w32.cu",
+           "stage1d.cu",
            "batch.cu", "static_batch.cu", "engine.cu", "server.cu", "tune.cu", "peaks.cu"]
-HEADERS = ["hweno_device.cuh", "launch.h", "server.h", "batch.h", "geometry.h",
-           "stage1d_item.cuh", "stage2d_item.cuh", "stage2d_char64.cuh", "stage2d_impl.cuh"]
+HEADERS = ["hweno_device.cuh", "f64_ops.cuh", "launch.h", "server.h", "batch.h", "geometry.h",
+           "stage1d_item.cuh", 
+           "stage2d_item.cuh", "recon64.cuh", "stage2d_char64.cuh",
+           "stage2d_comp64.cuh", "stage2d_tile64.cuh", "stage2d_impl.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
               "-I" + os.path.join(ROOT, "include")]

@@ -11,6 +11,8 @@
 // status); one thread per solve advances them at the start of each step, so each solve
 // steps with its own dt.  The work lists live in device memory: admission and retirement
 // rewrite them between steps and the captured step graph stays valid.
+#include <vector>
+
 #include "batch.h"
 #include "stage1d_item.cuh"
 #include "stage2d_item.cuh"
@@ -39,10 +41,10 @@ __global__ void batch_dt_kernel(BatchDt* d, BatchCtl* ctl, int nctl) {
 }
 
 template <int EQ, bool CHAR, typename R, int BW>
-__global__ void __launch_bounds__(BW, kMinBlocks2D<R, BW>)
+__global__ void __launch_bounds__(kThreads2D<R, BW>, kMinBlocks2D<EQ, R, BW>)
     batch_stage_kernel(const BatchSolve* bs, BatchCtl* ctl, int k) {
   extern __shared__ double smem[];
-  __shared__ double red[2][BW / 32];
+  __shared__ double red[2][kThreads2D<R, BW> / 32];
   __shared__ int item_s;
   const int n_items = ctl->n_items, n_solves = ctl->n_solves;
 #pragma unroll 1
@@ -136,7 +138,7 @@ static cudaError_t launch_batch1d_t(const BatchSolve* bs, BatchCtl* ctl, int k, 
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t init_batch_t(int* slots_out, size_t* local_out) {
-  constexpr int BW = kBatchBW;
+  constexpr int BW = batch_bw2d(sizeof(R) == 4);
   const size_t smem = smem_bytes2d<EQ, CHAR, R, BW>();
   auto kern = batch_stage_kernel<EQ, CHAR, R, BW>;
   static int slots = 0;
@@ -152,7 +154,7 @@ static cudaError_t init_batch_t(int* slots_out, size_t* local_out) {
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, BW, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads2D<R, BW>, smem);
     if (e != cudaSuccess) return e;
     slots = (per > 0 ? per : 1) * (nsm > 0 ? nsm : 1);
   }
@@ -163,11 +165,12 @@ static cudaError_t init_batch_t(int* slots_out, size_t* local_out) {
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t launch_batch_t(const BatchSolve* bs, BatchCtl* ctl, int k, cudaStream_t st) {
-  constexpr int BW = kBatchBW;
+  constexpr int BW = batch_bw2d(sizeof(R) == 4);
   int slots = 0;
   cudaError_t e = init_batch_t<EQ, CHAR, R>(&slots, nullptr);
   if (e != cudaSuccess) return e;
-  batch_stage_kernel<EQ, CHAR, R, BW><<<slots, BW, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(bs, ctl, k);
+  batch_stage_kernel<EQ, CHAR, R, BW>
+      <<<slots, kThreads2D<R, BW>, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(bs, ctl, k);
   return cudaGetLastError();
 }
 
@@ -259,11 +262,21 @@ int batch_slots(int cls) {
 
 void batch_geometry1d(int nx, int* blocks) { *blocks = (nx + (kBatchBW - 2) - 1) / (kBatchBW - 2); }
 
-void batch_geometry(int nx, int ny, int rows, int bw, int* bands, int* wout, int* chunks,
-                    bool lane_aware) {
-  split_bands(nx, default_bands(nx, bw, lane_aware), bands, wout);
+void batch_geometry(int nx, int ny, int rows, bool mixed, int* bands, int* wout, int* chunks) {
+  split_bands(nx, default_bands(nx, batch_bw2d(mixed), false), bands, wout);
   if (rows < 1) rows = 1;
   *chunks = (ny + rows - 1) / rows;
+}
+
+int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots) {
+  std::vector<int> bands(n), warps(n);
+  for (int s = 0; s < n; ++s) {
+    int wout, chunks;
+    batch_geometry(nx[s], ny[s], 1, mixed, &bands[s], &wout, &chunks);
+    warps[s] = (wout + 2 + 31) / 32;
+  }
+  return mixed ? batch_rows(bands.data(), ny, n, slots)
+               : batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX64, slots);
 }
 
 }  // namespace hw

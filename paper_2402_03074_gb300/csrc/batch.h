@@ -7,14 +7,15 @@
 
 namespace hw {
 
-// Threads per block of the batched stage kernels, every class.  The characteristic FP64 class
-// keeps the 128-thread kernel that forms the coefficients from each pass's projected stencil:
-// its 96-thread counterpart (coefficients once per cell, 111 KB of shared memory per block),
-// faster for a solve alone, shares the SMs worse with the FP32-bulk class's blocks of a mixed
-// stream (the configured served stream: 0.163 instead of 0.171 solves/s).  The FP32-bulk
-// class's 192-thread blocks, faster for a solve alone, have not been measured here.
+// Block width of the batched stage kernels: the FP32-bulk and 1D classes 128 threads (the
+// FP32-bulk class's 192-thread blocks, faster for a solve alone, have not been measured here),
+// the 2D FP64 classes tiles of 64 columns x 3 rows (against one row at a time in 128-thread
+// blocks, which hold only four warps per SM: a batch of eight solves of 200 x 184 to 284 x 261
+// cells, one step, 9.00 -> 7.58 ms; a served mix of six grids of 128^2 to 352^2 cells in both
+// precisions, 114 -> 95.5 ms).
 constexpr int kBatchBW = 128;
-inline int batch_bw2d(int, int, int) { return kBatchBW; }
+constexpr int kBatchBX64 = 64;
+constexpr int batch_bw2d(bool mixed) { return mixed ? kBatchBW : kBatchBX64; }
 constexpr int kBatchClasses = 16;  // {2D, 1D} x {advection, Burgers, Euler comp.-wise,
                                    // Euler char.} x {FP64, mixed}
 
@@ -47,11 +48,10 @@ struct BatchDt {
 };
 
 int batch_class(int equation, int characteristic, int mixed, int dim = 2);
-// bands (of at most bw - 2 columns for blocks of bw threads; lane_aware: of at most bw - 34
-// columns when that leaves fewer idle lanes, for the FP64 classes) and row chunks of `rows`
-// rows
-void batch_geometry(int nx, int ny, int rows, int bw, int* bands, int* wout, int* chunks,
-                    bool lane_aware = false);
+// bands of at most batch_bw2d() - 2 columns and row chunks of `rows` rows
+void batch_geometry(int nx, int ny, int rows, bool mixed, int* bands, int* wout, int* chunks);
+// rows per item for the 2D solves of one class (n grids) on `slots` resident blocks
+int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots);
 void batch_geometry1d(int nx, int* blocks);
 int batch_slots(int cls);  // resident blocks of the class's persistent launch
 cudaError_t launch_batch_dt(BatchDt* d, BatchCtl* ctl, int nctl, int cap, cudaStream_t st);

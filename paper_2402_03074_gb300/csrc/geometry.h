@@ -94,6 +94,91 @@ inline Geom2D geom2d(int nx, int ny, int bw, int slots, int rows_fixed, int band
   return g;
 }
 
+// ---- FP64 tiles: bx columns x tile_rows64(bx) rows of threads per block (stage2d_tile64.cuh),
+// six or seven warps, so that one block fills an SM's FP64 unit.
+constexpr int tile_rows64(int bx) { return bx == 32 ? 7 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
+
+// Time of a block in units of one row of one warp at the SM's full FP64 rate (16 clocks per warp
+// instruction): `warps` warps per row, `rows` output rows in `pieces` pieces, each with two ring
+// rows (0.46 of a row's work: the y pass without its volume sums); and at least 4.6 per step of
+// by rows, because a warp alone takes 64 clocks per FP64 instruction (and about 15 % more
+// for what its loads do not hide).
+inline double tile_time64(int warps, int by, int rows, int pieces) {
+  const double work = (double)warps * (rows + 0.92 * pieces);
+  const double steps = (double)((rows + 2 * pieces + by - 1) / by);
+  return work > 4.6 * steps ? work : 4.6 * steps;
+}
+
+// The default tile of an FP64 grid: over the widths bx[0..n-1] (with slots[] resident blocks per
+// GPU each, on `sms` SMs) and the chunk heights (or one segment per SM), the launch whose most
+// loaded SM is done first.  240^2: 32 x 7, 8 bands x 19 chunks of 13 rows (13.9, against 18.4 in
+// 96 x 2 tiles); 2048^2: 96 x 2, 22 bands in 152 segments of 297 band-rows (897, against 930 or
+// more in narrower bands, whose ring columns cost 3 and 7 % instead of 2 %).
+struct Tile64 {
+  int bx;
+  int rows;  // output rows per chunk; < -1: segments of -rows band-rows
+};
+inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* slots, int n) {
+  Tile64 best{96, 0};
+  double best_time = 1e300;
+  for (int q = 0; q < n; ++q) {
+    const int by = tile_rows64(bx[q]);
+    int bands, wout;
+    split_bands(nx, default_bands(nx, bx[q], false), &bands, &wout);
+    const int warps = (wout + 2 + 31) / 32;
+    auto consider = [&](long long blocks, int rows, int pieces, int encoded) {
+      const long long per_sm = (blocks + sms - 1) / sms;
+      const long long waves = (blocks + slots[q] - 1) / slots[q];
+      const double step = tile_time64(0, by, rows, pieces);   // the latency bound alone
+      const double work = (double)warps * (rows + 0.92 * pieces) * (double)per_sm;
+      const double time = work > step * (double)waves ? work : step * (double)waves;
+      if (time < 0.995 * best_time) {
+        best_time = time;
+        best = Tile64{bx[q], encoded};
+      }
+    };
+    for (int r = 1; r <= 16 && r <= ny; ++r) consider((long long)bands * ((ny + r - 1) / r), r, 1, r);
+    for (int m = 1; m <= 6; ++m) {
+      int c = m * sms / bands;
+      c = c < 1 ? 1 : (c > ny ? ny : c);
+      const int r = (ny + c - 1) / c;
+      consider((long long)bands * ((ny + r - 1) / r), r, 1, r);
+    }
+    const long long total = (long long)bands * ny;
+    const long long seg = (total + sms - 1) / sms;
+    if (bands <= sms && seg > 1)
+      consider((total + seg - 1) / seg, (int)seg, (int)(1 + (seg - 1 + ny - 1) / ny), -(int)seg);
+  }
+  return best;
+}
+
+// Rows per item of a batched FP64 class in tiles of bx columns (bands[s] bands of warps[s] warps
+// per row, ny[s] rows), whose persistent launch has `slots` resident blocks: the rows of least
+// waves x item time, the smallest (the most items) among equals.
+inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n, int bx,
+                        int slots) {
+  if (n <= 0 || slots <= 0) return 32;
+  int nymax = 1;
+  for (int s = 0; s < n; ++s) nymax = ny[s] > nymax ? ny[s] : nymax;
+  int best = 1;
+  double best_cost = 1e300;
+  for (int r = 1; r <= nymax; ++r) {
+    long long items = 0;
+    double time = 0.0;
+    for (int s = 0; s < n; ++s) {
+      items += (long long)bands[s] * ((ny[s] + r - 1) / r);
+      const double t = tile_time64(warps[s], tile_rows64(bx), r < ny[s] ? r : ny[s], 1);
+      time = t > time ? t : time;
+    }
+    const double cost = (double)((items + slots - 1) / slots) * time;
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = r;
+    }
+  }
+  return best;
+}
+
 // Rows per work item for the 2D solves of one batched class (bands[s] bands and ny[s] rows
 // each) whose persistent launch has `slots` resident blocks.  The launch runs
 // ceil(items / slots) waves, a partial last wave costing a whole item time, and an item costs

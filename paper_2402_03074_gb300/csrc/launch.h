@@ -70,12 +70,12 @@ struct TileShape {
   int width = 0;
   int lanes = 0;
 };
-// Default block width of the 2D single-solve launch: 96 threads for characteristic FP64
-// Euler (the kernel that keeps the conserved coefficients in shared memory), 192 for
-// characteristic FP32-bulk Euler (two blocks per SM: fewer idle lanes and ring columns than
-// three of 128; 8.3 ms instead of 9.1 ms per 2048^2 stage), else 128.
+// Default block width of the 2D single-solve launch: for the FP64 classes 96 columns (with the
+// default geometry the tile is then chosen for the grid, geometry.h), 192 for characteristic
+// FP32-bulk Euler (two blocks per SM: fewer idle lanes and ring columns than three of 128;
+// 8.3 ms instead of 9.1 ms per 2048^2 stage), else 128.
 constexpr int default_width2d(int eq, bool characteristic, bool mixed) {
-  return eq == EQ_EULER && characteristic ? (mixed ? 192 : 96) : 128;
+  return !mixed ? 96 : (eq == EQ_EULER && characteristic ? 192 : 128);
 }
 // Tuning table keyed by (equation, characteristic, precision, nx, ny); all zero = not tuned.
 TileShape tuning_shape(int eq, int characteristic, int mixed, int nx, int ny);

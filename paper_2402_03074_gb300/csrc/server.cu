@@ -155,23 +155,19 @@ static int rebuild_lists(Server* S, cudaStream_t st, unsigned* classes) {
   // rows per work item, per class: the fewest waves of items over the class's resident
   // block slots for the length of its launch (a partial last wave costs a whole item time;
   // taller items waste fewer ring rows, but fewer items than slots leave SMs idle)
-  std::vector<int> cb[kBatchClasses], cy[kBatchClasses];
+  std::vector<int> cx[kBatchClasses], cy[kBatchClasses];
   for (Request* r : S->live) {
     const hweno_problem* p = solve_problem(r->solve);
     if (!batched(p) || p->dim != 2) continue;
     const int cls = class_of(p);
-    int bands, wout, chunks;
-    batch_geometry(p->nx, p->ny, 1,
-                   batch_bw2d(p->equation, p->characteristic, p->precision == HWENO_MIXED32),
-                   &bands, &wout, &chunks, p->precision != HWENO_MIXED32);
-    cb[cls].push_back(bands);
+    cx[cls].push_back(p->nx);
     cy[cls].push_back(p->ny);
   }
   int rows_of[kBatchClasses];
   for (int c = 0; c < kBatchClasses; ++c)
-    rows_of[c] = cb[c].empty() ? S->rows
-                               : batch_rows(cb[c].data(), cy[c].data(), (int)cb[c].size(),
-                                            batch_slots(c));
+    rows_of[c] = cx[c].empty() ? S->rows
+                               : batch_item_rows(cx[c].data(), cy[c].data(), (int)cx[c].size(),
+                                                 (c & 1) != 0, batch_slots(c));
   int n = 0, nall = 0;
   *classes = 0;
   for (Request* r : S->live) {
@@ -193,8 +189,7 @@ static int rebuild_lists(Server* S, cudaStream_t st, unsigned* classes) {
     B.mixed = p->precision == HWENO_MIXED32;
     if (p->dim == 2) {
       B.rows = rows_of[cls];
-      batch_geometry(p->nx, p->ny, B.rows, batch_bw2d(p->equation, p->characteristic, B.mixed),
-                     &B.bands, &B.wout, &B.chunks, !B.mixed);
+      batch_geometry(p->nx, p->ny, B.rows, B.mixed != 0, &B.bands, &B.wout, &B.chunks);
     } else {
       batch_geometry1d(p->nx, &B.bands);
       B.wout = kBatchBW - 2;

@@ -13,11 +13,11 @@ namespace hw {
 // segments, block b sweeping the band-rows [b seg, (b + 1) seg) of the `bands` bands taken one
 // after another, in one piece per band it touches
 template <int EQ, bool CHAR, typename R, int BW>
-__global__ void __launch_bounds__(BW, kMinBlocks2D<R, BW>)
+__global__ void __launch_bounds__(kThreads2D<R, BW>, kMinBlocks2D<EQ, R, BW>)
     stage2d_kernel(KProblem P, KStage S, int rows, int wout, int seg, int bands) {
   if (S.active && *S.active == 0) return;
   extern __shared__ double smem[];
-  __shared__ double red[2][BW / 32];
+  __shared__ double red[2][kThreads2D<R, BW> / 32];
   const int ny = P.ny;
   // the block's pieces: one (band, row chunk), or the pieces of its segment; one call site of
   // the (large, inlined) work item
@@ -63,7 +63,7 @@ static cudaError_t init2d_t(int* slots_out, size_t* local_out) {
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, BW, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads2D<R, BW>, smem);
     if (e != cudaSuccess) return e;
     slots = (per > 0 ? per : 1) * (nsm > 0 ? nsm : 1);
   }
@@ -80,9 +80,9 @@ static cudaError_t launch2d_w(const KProblem& P, const KStage& S, TileShape t, c
   // bands of equal width, swept in row chunks or segments filling the resident block slots
   // once, unless the tuning table (or the autotuner) fixes the tile shape (geometry.h)
   const Geom2D g = geom2d(P.nx, P.ny, BW, slots, (t.rows > 0 || t.rows < -1) ? t.rows : 0,
-                          t.bands > 0 ? t.bands : 0, sizeof(R) == sizeof(double));
+                          t.bands > 0 ? t.bands : 0, false);
   const dim3 grid = g.seg > 0 ? dim3(g.blocks) : dim3(g.bands, g.chunks);
-  stage2d_kernel<EQ, CHAR, R, BW><<<grid, BW, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(
+  stage2d_kernel<EQ, CHAR, R, BW><<<grid, kThreads2D<R, BW>, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(
       P, S, g.rows, g.wout, g.seg, g.bands);
   return cudaGetLastError();
 }
@@ -94,19 +94,57 @@ cudaError_t launch2d_width(int eq, bool characteristic, bool mixed, const KProbl
                            const KStage& S, TileShape t, cudaStream_t st);
 template <int BW>
 cudaError_t prepare2d_width(size_t* max_local);
+// resident blocks per GPU of the class's FP64 kernel in tiles BW columns wide
+template <int BW>
+cudaError_t slots64_width(int eq, bool characteristic, int* slots);
 #define HW_STAGE2D_DECLARE(BW)                                                                \
   template <>                                                                                 \
   cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool mixed, const KProblem& P,  \
                                  const KStage& S, TileShape t, cudaStream_t st);              \
   template <>                                                                                 \
-  cudaError_t prepare2d_width<BW>(size_t* max_local);
+  cudaError_t prepare2d_width<BW>(size_t* max_local);                                         \
+  template <>                                                                                 \
+  cudaError_t slots64_width<BW>(int eq, bool characteristic, int* slots);
+HW_STAGE2D_DECLARE(32)
 HW_STAGE2D_DECLARE(128)
 HW_STAGE2D_DECLARE(96)
 HW_STAGE2D_DECLARE(64)
 HW_STAGE2D_DECLARE(192)
 #undef HW_STAGE2D_DECLARE
 
+// the FP64 classes of one width
+#define HW_STAGE2D_SLOTS64(BW)                                                                \
+  template <>                                                                                 \
+  cudaError_t slots64_width<BW>(int eq, bool characteristic, int* slots) {                    \
+    if (eq == EQ_ADV) return init2d_t<EQ_ADV, false, double, BW>(slots, nullptr);             \
+    if (eq == EQ_BURG) return init2d_t<EQ_BURG, false, double, BW>(slots, nullptr);           \
+    if (characteristic) return init2d_t<EQ_EULER, true, double, BW>(slots, nullptr);          \
+    return init2d_t<EQ_EULER, false, double, BW>(slots, nullptr);                             \
+  }
+#define HW_STAGE2D_WIDTH64(BW)                                                                \
+  HW_STAGE2D_SLOTS64(BW)                                                                      \
+  template <>                                                                                 \
+  cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool, const KProblem& P,        \
+                                 const KStage& S, TileShape t, cudaStream_t st) {             \
+    if (eq == EQ_ADV) return launch2d_w<EQ_ADV, false, double, BW>(P, S, t, st);              \
+    if (eq == EQ_BURG) return launch2d_w<EQ_BURG, false, double, BW>(P, S, t, st);            \
+    if (characteristic) return launch2d_w<EQ_EULER, true, double, BW>(P, S, t, st);           \
+    return launch2d_w<EQ_EULER, false, double, BW>(P, S, t, st);                              \
+  }                                                                                           \
+  template <>                                                                                 \
+  cudaError_t prepare2d_width<BW>(size_t* max_local) {                                        \
+    size_t m = 0, l = 0;                                                                      \
+    cudaError_t e = init2d_t<EQ_ADV, false, double, BW>(nullptr, &m);                         \
+    if (e == cudaSuccess && (e = init2d_t<EQ_BURG, false, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;   \
+    if (e == cudaSuccess && (e = init2d_t<EQ_EULER, false, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;  \
+    if (e == cudaSuccess && (e = init2d_t<EQ_EULER, true, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;   \
+    if (max_local) *max_local = m;                                                            \
+    return e;                                                                                 \
+  }
+
+// every class of one width
 #define HW_STAGE2D_WIDTH(BW)                                                                  \
+  HW_STAGE2D_SLOTS64(BW)                                                                      \
   template <>                                                                                 \
   cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool mixed, const KProblem& P,  \
                                  const KStage& S, TileShape t, cudaStream_t st) {             \

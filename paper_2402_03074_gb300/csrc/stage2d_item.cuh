@@ -12,19 +12,27 @@
 // and the wave speed of the output is folded into a block maximum.  Redundant work is the
 // two ring columns per band and the two ring rows per chunk (x pass skipped on ring rows).
 #pragma once
+#include "geometry.h"
 #include "hweno_device.cuh"
-#include "stage2d_char64.cuh"
+#include "stage2d_tile64.cuh"
 
 namespace hw {
 
 
-// Resident blocks per SM the 2D stage kernels are compiled for: the FP64 kernels take the
-// whole register file at 255 registers per thread (one 128- or 192-thread block, two of 96
-// threads, four of 64), the FP32-bulk kernels twelve warps (at most 168 registers per thread:
-// two 192-thread, three 128-thread, four 96-thread or six 64-thread blocks), which hides more
-// of the FP64 latency of their weight evaluation.
+// Threads of a block: bands of at most BW - 2 columns, one row at a time in the FP32-bulk
+// kernels, tile_rows64(BW) rows at once in the FP64 ones.
+template <int BW>
+constexpr int kTileRows64 = tile_rows64(BW);
 template <typename R, int BW>
-constexpr int kMinBlocks2D = sizeof(R) == 4 ? 384 / BW : (BW == 128 ? 1 : 256 / BW);
+constexpr int kThreads2D = sizeof(R) == sizeof(double) ? BW * kTileRows64<BW> : BW;
+
+// Resident blocks per SM the 2D stage kernels are compiled for: the FP64 Euler kernels take the
+// register file and the shared memory with one block (two of 128 threads would not fit), the
+// scalar FP64 ones two; the FP32-bulk kernels twelve warps (at most 168 registers per thread: two
+// 192-thread, three 128-thread, four 96-thread or six 64-thread blocks), which hides more of
+// the FP64 latency of their weight evaluation.
+template <int EQ, typename R, int BW>
+constexpr int kMinBlocks2D = sizeof(R) == sizeof(double) ? (EQ == EQ_EULER ? 1 : 2) : 384 / BW;
 
 // Gauss weights on [-1/2, 1/2] (sum 1) and nodes
 #define GW0 (5.0 / 18.0)
@@ -61,29 +69,22 @@ __device__ __forceinline__ void volume_sum(const KProblem& P, int dir, const R (
 // when a row is loaded); the FP64 update reads the cell's own averages from global memory
 // when R is float.
 
-// Characteristic FP64 Euler has an item of its own (stage2d_char64.cuh).
-template <int EQ, bool CHAR, typename R>
-constexpr bool kChar64 = EQ == EQ_EULER && CHAR && sizeof(R) == sizeof(double);
-
 // Shared memory of a block: the 3-row window, the x-face exchange and the top traces carried
 // from row to row (in shared memory rather than in 48 registers: fewer spills, FP32-bulk
 // stages 2 % faster).
 template <int EQ, bool CHAR, typename R, int BW>
 constexpr size_t smem_bytes2d() {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
-  if constexpr (kChar64<EQ, CHAR, R>) return smem_bytes_char64<BW>();
+  if constexpr (sizeof(R) == sizeof(double))
+    return smem_bytes_tile64<EQ, CHAR, BW, kTileRows64<BW>>();
   return sizeof(R) * 3 * NC * 3 * (BW + 2) + sizeof(R) * NC * 3 * 2 * BW +
          sizeof(R) * 2 * 3 * NC * BW;
 }
 
 template <int EQ, bool CHAR, typename R, int BW>
-__device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S, int band,
-                                             int j0, int j1, int wout, double* smem,
-                                             double (*red)[BW / 32]) {
-  if constexpr (kChar64<EQ, CHAR, R>) {
-    stage2d_char64_item<BW>(P, S, band, j0, j1, wout, smem, red);
-    return;
-  }
+__device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KStage& S, int band,
+                                                   int j0, int j1, int wout, double* smem,
+                                                   double (*red)[BW / 32]) {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
   constexpr int NM = 3;
   constexpr int NA = NC * NM;
@@ -512,6 +513,17 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
     atomic_max_nonneg(&S.alpha_out[1], m1);
   }
   __syncthreads();  // the block may start another item in the same shared memory
+}
+
+// One work item of the class.
+template <int EQ, bool CHAR, typename R, int BW>
+__device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S, int band,
+                                             int j0, int j1, int wout, double* smem,
+                                             double (*red)[kThreads2D<R, BW> / 32]) {
+  if constexpr (sizeof(R) == sizeof(double))
+    stage2d_tile64_item<EQ, CHAR, BW, kTileRows64<BW>>(P, S, band, j0, j1, wout, smem, red);
+  else
+    stage2d_mixed_item<EQ, CHAR, R, BW>(P, S, band, j0, j1, wout, smem, red);
 }
 
 }  // namespace hw

@@ -59,10 +59,10 @@ __global__ void static_setup_kernel(StaticScratch* dst, StaticScratch src) {
 }
 
 template <int EQ, bool CHAR, typename R, int BW>
-__global__ void __launch_bounds__(BW, kMinBlocks2D<R, BW>)
+__global__ void __launch_bounds__(kThreads2D<R, BW>, kMinBlocks2D<EQ, R, BW>)
     static_batch_kernel(StaticScratch* sc, int k) {
   extern __shared__ double smem[];
-  __shared__ double red[2][BW / 32];
+  __shared__ double red[2][kThreads2D<R, BW> / 32];
   __shared__ int item_s;
   const int n_items = sc->n_items, n = sc->n;
 #pragma unroll 1
@@ -109,7 +109,7 @@ static bool g_static_ready[64];
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t static_class_setup(int* slots, size_t* local) {
-  constexpr int BW = kBatchBW;
+  constexpr int BW = batch_bw2d(sizeof(R) == 4);
   auto kern = static_batch_kernel<EQ, CHAR, R, BW>;
   const size_t smem = smem_bytes2d<EQ, CHAR, R, BW>();
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -121,7 +121,7 @@ static cudaError_t static_class_setup(int* slots, size_t* local) {
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, BW, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads2D<R, BW>, smem);
   if (e != cudaSuccess) return e;
   *slots = (per > 0 ? per : 1) * (nsm > 0 ? nsm : 1);
   return cudaSuccess;
@@ -129,8 +129,9 @@ static cudaError_t static_class_setup(int* slots, size_t* local) {
 
 template <int EQ, bool CHAR, typename R>
 static void static_launch(int slots, StaticScratch* ptr, int k, cudaStream_t st) {
-  constexpr int BW = kBatchBW;
-  static_batch_kernel<EQ, CHAR, R, BW><<<slots, BW, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(ptr, k);
+  constexpr int BW = batch_bw2d(sizeof(R) == 4);
+  static_batch_kernel<EQ, CHAR, R, BW>
+      <<<slots, kThreads2D<R, BW>, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(ptr, k);
 }
 
 // set-up of one device (the current one): scratch address and every class's launch setup
@@ -210,16 +211,13 @@ extern "C" int hweno_stage_batch_static(int n, const hweno_problem* problems, in
   // waves of items over the resident block slots for its length
   StaticScratch host;
   std::memset(&host, 0, sizeof(host));
-  int bands[HWENO_STATIC_BATCH_MAX], wout[HWENO_STATIC_BATCH_MAX], chunks[HWENO_STATIC_BATCH_MAX];
-  int nys[HWENO_STATIC_BATCH_MAX];
+  const bool mixed = p0.precision == HWENO_MIXED32;
+  int nxs[HWENO_STATIC_BATCH_MAX], nys[HWENO_STATIC_BATCH_MAX];
   for (int s = 0; s < n; ++s) {
-    batch_geometry(problems[s].nx, problems[s].ny, 1,
-                   batch_bw2d(problems[s].equation, problems[s].characteristic,
-                              problems[s].precision == HWENO_MIXED32),
-                   &bands[s], &wout[s], &chunks[s]);
+    nxs[s] = problems[s].nx;
     nys[s] = problems[s].ny;
   }
-  const int rows = batch_rows(bands, nys, n, D.slots[cls]);
+  const int rows = batch_item_rows(nxs, nys, n, mixed, D.slots[cls]);
   int items = 0;
   for (int s = 0; s < n; ++s) {
     StaticItem& it = host.item[s];
@@ -232,10 +230,8 @@ extern "C" int hweno_stage_batch_static(int n, const hweno_problem* problems, in
     it.alpha_out = alpha_out[s];
     it.dt = dt[s];
     it.status = status[s];
-    it.bands = bands[s];
-    it.wout = wout[s];
     it.rows = rows;
-    it.chunks = (problems[s].ny + it.rows - 1) / it.rows;
+    batch_geometry(nxs[s], nys[s], rows, mixed, &it.bands, &it.wout, &it.chunks);
     it.item_base = items;
     items += it.bands * it.chunks;
   }
