@@ -14,7 +14,7 @@
 #include <vector>
 
 #include "batch.h"
-#include "stage1d_item.cuh"
+#include "stage1d_lanes64.cuh"
 #include "stage2d_item.cuh"
 
 namespace hw {
@@ -78,6 +78,7 @@ template <int EQ, bool CHAR, typename R, int BW>
 __global__ void __launch_bounds__(BW) batch1d_stage_kernel(const BatchSolve* bs, BatchCtl* ctl,
                                                            int k) {
   __shared__ int item_s;
+  __shared__ double tab[l64::kTable];
   const int n_items = ctl->n_items, n_solves = ctl->n_solves;
 #pragma unroll 1
   for (;;) {
@@ -99,7 +100,8 @@ __global__ void __launch_bounds__(BW) batch1d_stage_kernel(const BatchSolve* bs,
     S.status = &B.sc->status;
     S.active = &B.sc->active;
     S.k = k;
-    stage1d_item<EQ, CHAR, R, BW>(B.P, S, item - B.item_base);
+    if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, B.P);
+    thread_item1d<EQ, CHAR, R, BW>(B.P, S, item - B.item_base, tab);
   }
 }
 

@@ -763,6 +763,16 @@ struct Eig2 {
   }
 };
 
+// the largest of the warp's non-negative doubles (their bits in value order), in two integer
+// reductions (a double maximum costs an FP64 instruction per shuffle)
+__device__ __forceinline__ double warp_max_nonneg(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32);
+  const unsigned m = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)b : 0u);
+  return __longlong_as_double((long long)((unsigned long long)m << 32 | lo));
+}
+
 // atomic max of a non-negative double (bit pattern order = value order for x >= 0)
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
   if (!(v >= 0.0)) v = __longlong_as_double(0x7ff0000000000000ULL);  // NaN -> +inf

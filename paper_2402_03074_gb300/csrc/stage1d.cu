@@ -1,15 +1,19 @@
 // stage1d.cu -- single-solve launch of the fused 1D HWENO-U stage (one block per BW-2 cells;
 // the block's work is in stage1d_item.cuh).
 //
-// Block width: a stage is FP64-pipe bound per SM, and an SM has one FP64 unit however many of
-// a grid's blocks it holds, so a short grid must be spread over as many SMs as possible.  The
-// 128-thread blocks (126 cells each) are used once they give every SM at least one block;
-// shorter grids take one-warp blocks of 30 cells (4000 cells: 134 blocks on 134 SMs instead of
-// 32 blocks on 32 SMs).
+// Layout: a warp gets one FP64 instruction in 64 clocks however few of its lanes are active, and
+// an SM runs four warps at that rate, so a short grid is bound by the FP64 instructions of one
+// warp.  FP64 solves of at most 30 cells per SM (4560 on 152 SMs) take four lanes per cell in
+// 128-thread blocks of 30 cells (stage1d_lanes64.cuh), one block per SM; beyond that more than
+// four warps share an SM and the lanes' redundant work costs more than it saves, and one thread
+// per cell is used: 128-thread blocks (126 cells each) once they give every SM at least one
+// block, else one-warp blocks of 30 cells.  FP32-bulk solves: one thread per cell, and one lane
+// per characteristic field for Euler grids that fit a cluster.
 #include <cooperative_groups.h>
 
 #include "launch.h"
 #include "stage1d_item.cuh"
+#include "stage1d_lanes64.cuh"
 
 namespace hw {
 
@@ -34,38 +38,54 @@ static int sm_count() {
 template <int EQ, bool CHAR, typename R, int BW>
 __global__ void __launch_bounds__(BW) stage1d_kernel(KProblem P, KStage S) {
   if (S.active && *S.active == 0) return;
-  stage1d_item<EQ, CHAR, R, BW>(P, S, blockIdx.x);
+  __shared__ double tab[l64::kTable];
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, P);
+  thread_item1d<EQ, CHAR, R, BW>(P, S, blockIdx.x, tab);
 }
 
-template <typename R, int BW>
-__global__ void __launch_bounds__(BW) stage1d_fields_kernel(KProblem P, KStage S) {
+// classes with a layout of four lanes per cell
+template <int EQ, bool CHAR, typename R>
+constexpr bool kLanes1D = sizeof(R) == sizeof(double) || (EQ == EQ_EULER && CHAR);
+
+// one block of the four-lanes layout; tab: the FP64 table of constants, filled by the block
+template <int EQ, bool CHAR, typename R, int BW, class IO>
+__device__ __forceinline__ void lanes_item(const KProblem& P, const IO& io, int blk, double* tab) {
+  if constexpr (sizeof(R) == sizeof(double)) stage1d_lanes64_item_io<EQ, CHAR, BW>(P, io, blk, tab);
+  else stage1d_fields_item_io<R, BW>(P, io, blk);
+}
+
+template <int EQ, bool CHAR, typename R, int BW>
+__global__ void __launch_bounds__(BW) stage1d_lanes_kernel(KProblem P, KStage S) {
   if (S.active && *S.active == 0) return;
-  stage1d_fields_item<R, BW>(P, S, blockIdx.x);
+  __shared__ double tab[l64::kTable];
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, P);
+  const Global1D io{S, P.nx};
+  lanes_item<EQ, CHAR, R, BW>(P, io, blockIdx.x, tab);
 }
 
 template <int EQ, bool CHAR, typename R>
-static bool short_fields1d(int nx);
+static bool default_lanes1d(int nx);
 
 // blocks of BW threads, BW - 2 cells each (one thread per cell), or BW / 4 - 2 cells each
-// (one lane per characteristic field)
+// (four lanes per cell)
 template <int EQ, bool CHAR, typename R>
 static cudaError_t launch1d_t(const KProblem& P, const KStage& S, cudaStream_t st) {
   TileShape ts;
   if (g_force1d.width || g_force1d.lanes) ts = g_force1d;
   else ts = tuning_shape(EQ, CHAR ? 1 : 0, sizeof(R) == 4 ? 1 : 0, P.nx, 1);
-  if (ts.width == 0 && ts.lanes == 0 && short_fields1d<EQ, CHAR, R>(P.nx)) {
+  if (ts.width == 0 && ts.lanes == 0 && default_lanes1d<EQ, CHAR, R>(P.nx)) {
     ts.width = 128;
     ts.lanes = 4;
   }
-  if constexpr (EQ == EQ_EULER && CHAR) {
+  if constexpr (kLanes1D<EQ, CHAR, R>) {
     if (ts.lanes == 4) {
       const int w = ts.width ? ts.width : 128;
       if (w == 32)
-        stage1d_fields_kernel<R, 32><<<(P.nx + 5) / 6, 32, 0, st>>>(P, S);
+        stage1d_lanes_kernel<EQ, CHAR, R, 32><<<(P.nx + 5) / 6, 32, 0, st>>>(P, S);
       else if (w == 64)
-        stage1d_fields_kernel<R, 64><<<(P.nx + 13) / 14, 64, 0, st>>>(P, S);
+        stage1d_lanes_kernel<EQ, CHAR, R, 64><<<(P.nx + 13) / 14, 64, 0, st>>>(P, S);
       else
-        stage1d_fields_kernel<R, 128><<<(P.nx + 29) / 30, 128, 0, st>>>(P, S);
+        stage1d_lanes_kernel<EQ, CHAR, R, 128><<<(P.nx + 29) / 30, 128, 0, st>>>(P, S);
       return cudaGetLastError();
     }
   }
@@ -86,9 +106,11 @@ static cudaError_t launch1d_t(const KProblem& P, const KStage& S, cudaStream_t s
 // non-physical state).  Every cell is computed by the same item code as in the per-stage
 // launches, so the results are bitwise those of the graph-replayed steps; a step costs one
 // grid barrier per stage instead of four launches.
-template <int EQ, bool CHAR, typename R, int BW, bool FIELDS>
+template <int EQ, bool CHAR, typename R, int BW, bool LANES>
 __global__ void __launch_bounds__(BW) step1d_coop_kernel(Step1D A, int nsteps, int items) {
   cg::grid_group grid = cg::this_grid();
+  __shared__ double tab[l64::kTable];
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, A.P);
   volatile int* active = &A.sc->active;
 #pragma unroll 1
   for (int s = 0; s < nsteps; ++s) {
@@ -110,8 +132,8 @@ __global__ void __launch_bounds__(BW) step1d_coop_kernel(Step1D A, int nsteps, i
       S.k = k;
 #pragma unroll 1
       for (int it = blockIdx.x; it < items; it += gridDim.x) {
-        if constexpr (FIELDS) stage1d_fields_item<R, BW>(A.P, S, it);
-        else stage1d_item<EQ, CHAR, R, BW>(A.P, S, it);
+        if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, Global1D{S, A.P.nx}, it, tab);
+        else thread_item1d<EQ, CHAR, R, BW>(A.P, S, it, tab);
       }
       grid.sync();
     }
@@ -189,6 +211,7 @@ __device__ __forceinline__ void cluster_reduce(DevScal& sc, double (*amax)[1], u
                                                int k, int nb) {
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   const int t = threadIdx.x;
+  if (t >= 32) return;
   double v = 0.0;
   unsigned b = 0u;
   if (t < nb) {
@@ -196,37 +219,35 @@ __device__ __forceinline__ void cluster_reduce(DevScal& sc, double (*amax)[1], u
     if (!(v >= 0.0)) v = __longlong_as_double(0x7ff0000000000000LL);  // NaN -> +inf
     b = cl.map_shared_rank(&bad[k][0], t)[0];
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    b |= __shfl_xor_sync(0xffffffffu, b, o);
-  }
+  v = warp_max_nonneg(v);
+  b = __reduce_or_sync(0xffffffffu, b);
   if (t == 0) {
-    sc.alpha[k][0] = fmax(sc.alpha[k][0], v);
+    sc.alpha[k][0] = v;  // cleared at the start of the step
     if (b) sc.status |= kStatusNonphysical;
   }
 }
 
-// CTA width of the cluster kernel: one warp (one thread per cell), or 128 threads for one
-// lane per characteristic field (32 cell slots, 1D Euler with the characteristic
-// decomposition); either way a CTA owns kClusterW cells and its item window has
+// CTA width of the cluster kernel: one warp (one thread per cell), or 128 threads for four
+// lanes per cell (32 cell slots); either way a CTA owns kClusterW cells and its item window has
 // kClusterW + 4 columns.
-template <bool FIELDS>
-constexpr int kClusterBW = FIELDS ? 128 : 32;
+template <bool LANES>
+constexpr int kClusterBW = LANES ? 128 : 32;
 
-template <int EQ, bool CHAR, typename R, bool FIELDS>
-__global__ void __launch_bounds__(kClusterBW<FIELDS>) step1d_cluster_kernel(Step1D A,
+template <int EQ, bool CHAR, typename R, bool LANES>
+__global__ void __launch_bounds__(kClusterBW<LANES>) step1d_cluster_kernel(Step1D A,
                                                                           int nsteps) {
-  constexpr int BW = kClusterBW<FIELDS>, W = kClusterW, NC = (EQ == EQ_EULER) ? 3 : 1;
+  constexpr int BW = kClusterBW<LANES>, W = kClusterW, NC = (EQ == EQ_EULER) ? 3 : 1;
   constexpr int NA = NC * 2, WC = W + 4;
   constexpr int SL = (NA * WC + BW - 1) / BW;  // window entries per thread
-  static_assert(FIELDS ? (W == BW / 4 - 2) : (W == BW - 2), "a CTA owns its item's cells");
+  static_assert(LANES ? (W == BW / 4 - 2) : (W == BW - 2), "a CTA owns its item's cells");
   cg::cluster_group cl = cg::this_cluster();
   __shared__ double st[3][NA][W];
   __shared__ double vhs[NC][W];
   __shared__ double amax[4][1];   // [k]: this CTA's maximum output speed of stage k
   __shared__ unsigned bad[4][1];  // [k]: this CTA's non-physical flag of stage k
   __shared__ DevScal scl;         // the solve's scalars (every CTA holds the same values)
+  __shared__ double ctab[l64::kTable];
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(ctab, A.P);
   const int rank = (int)cl.block_rank(), nb = (int)cl.num_blocks();
   const int nx = A.P.nx, i0 = rank * W, t = threadIdx.x;
   for (int q = t; q < NA * W; q += BW) {
@@ -275,7 +296,7 @@ __global__ void __launch_bounds__(kClusterBW<FIELDS>) step1d_cluster_kernel(Step
       Cluster1D<NA, W, SL, R> io{st, vhs, &amax[k][0], &bad[k][0], &tab, k - 1, k % 3, k, i0,
                                  scl.dt, scl.alpha[k - 1][0]};
       if (t == 0) bad[k][0] = 0u;
-      if constexpr (FIELDS) stage1d_fields_item_io<R, BW>(A.P, io, rank);
+      if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, io, rank, ctab);
       else stage1d_item_io<EQ, CHAR, R, BW>(A.P, io, rank);
     }
   }
@@ -289,7 +310,7 @@ __global__ void __launch_bounds__(kClusterBW<FIELDS>) step1d_cluster_kernel(Step
 
 // Largest cluster (CTAs) the device runs for this kernel: 16 where non-portable cluster sizes
 // are allowed and a 16-CTA cluster fits, else 8; 0 if clusters are not available.
-template <int EQ, bool CHAR, typename R, bool FIELDS>
+template <int EQ, bool CHAR, typename R, bool LANES>
 static int cluster_max() {
   static int cache[64] = {};
   int dev = 0;
@@ -299,13 +320,13 @@ static int cluster_max() {
   cudaDeviceGetAttribute(&cc, cudaDevAttrComputeCapabilityMajor, dev);
   int best = -1;
   if (cc >= 9) {
-    auto kern = step1d_cluster_kernel<EQ, CHAR, R, FIELDS>;
+    auto kern = step1d_cluster_kernel<EQ, CHAR, R, LANES>;
     best = 8;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
         cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(16);
-      cfg.blockDim = dim3(kClusterBW<FIELDS>);
+      cfg.blockDim = dim3(kClusterBW<LANES>);
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = 16;
@@ -322,11 +343,11 @@ static int cluster_max() {
   return best > 0 ? best : 0;
 }
 
-template <int EQ, bool CHAR, typename R, bool FIELDS>
+template <int EQ, bool CHAR, typename R, bool LANES>
 static cudaError_t cluster_launch(const Step1D& A, int nsteps, int nb, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nb);
-  cfg.blockDim = dim3(kClusterBW<FIELDS>);
+  cfg.blockDim = dim3(kClusterBW<LANES>);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -336,27 +357,29 @@ static cudaError_t cluster_launch(const Step1D& A, int nsteps, int nb, cudaStrea
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, step1d_cluster_kernel<EQ, CHAR, R, FIELDS>, A, nsteps);
+  return cudaLaunchKernelEx(&cfg, step1d_cluster_kernel<EQ, CHAR, R, LANES>, A, nsteps);
 }
 
-// 1D Euler with the characteristic decomposition on a grid short enough for one cluster: the
-// default layout (no tuning-table entry) is one lane per characteristic field in 128-thread
-// blocks of 30 cells, in the per-stage, the cooperative and the cluster-resident launches
-// alike (so hweno_step and hweno_advance give the same bits).
+// The grids whose default layout (no tuning-table entry) is four lanes per cell in 128-thread
+// blocks of 30 cells, in the per-stage, the cooperative and the cluster-resident launches alike
+// (so hweno_step and hweno_advance give the same bits): FP64 solves of at most one such block per
+// SM; FP32-bulk Euler with the characteristic decomposition on a grid short enough for one
+// cluster.
 template <int EQ, bool CHAR, typename R>
-static bool short_fields1d(int nx) {
-  if constexpr (EQ == EQ_EULER && CHAR) {
-    const int m = cluster_max<EQ, CHAR, R, true>();
-    return m > 0 && (nx + kClusterW - 1) / kClusterW <= m;
+static bool default_lanes1d(int nx) {
+  const int blocks = (nx + kClusterW - 1) / kClusterW;
+  if constexpr (sizeof(R) == sizeof(double)) {
+    return blocks <= sm_count();
+  } else if constexpr (EQ == EQ_EULER && CHAR) {
+    return blocks <= cluster_max<EQ, CHAR, R, true>();
   } else {
-    (void)nx;
     return false;
   }
 }
 
-template <int EQ, bool CHAR, typename R, int BW, bool FIELDS>
+template <int EQ, bool CHAR, typename R, int BW, bool LANES>
 static cudaError_t coop_launch(const Step1D& A, int nsteps, int items, cudaStream_t st) {
-  auto kern = step1d_coop_kernel<EQ, CHAR, R, BW, FIELDS>;
+  auto kern = step1d_coop_kernel<EQ, CHAR, R, BW, LANES>;
   static int per_sm = 0;
   if (per_sm == 0) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BW, 0);
@@ -378,18 +401,22 @@ static cudaError_t steps1d_t(const Step1D& A, int nsteps, cudaStream_t st) {
   // back to the cooperative launch of the same layout)
   const int nb = (nx + kClusterW - 1) / kClusterW;
   const bool untuned = ts.width == 0 && ts.lanes == 0;
-  if constexpr (EQ == EQ_EULER && CHAR) {
-    if (untuned && short_fields1d<EQ, CHAR, R>(nx)) {
-      if (cluster_launch<EQ, CHAR, R, true>(A, nsteps, nb, st) == cudaSuccess) return cudaSuccess;
-      cudaGetLastError();
+  if constexpr (kLanes1D<EQ, CHAR, R>) {
+    if (untuned && default_lanes1d<EQ, CHAR, R>(nx)) {
+      if (nb <= cluster_max<EQ, CHAR, R, true>()) {
+        if (cluster_launch<EQ, CHAR, R, true>(A, nsteps, nb, st) == cudaSuccess) return cudaSuccess;
+        cudaGetLastError();
+      }
       return coop_launch<EQ, CHAR, R, 128, true>(A, nsteps, (nx + 29) / 30, st);
     }
   }
-  if (untuned && nb <= cluster_max<EQ, CHAR, R, false>()) {
-    if (cluster_launch<EQ, CHAR, R, false>(A, nsteps, nb, st) == cudaSuccess) return cudaSuccess;
-    cudaGetLastError();
+  if constexpr (sizeof(R) == sizeof(float)) {
+    if (untuned && nb <= cluster_max<EQ, CHAR, R, false>()) {
+      if (cluster_launch<EQ, CHAR, R, false>(A, nsteps, nb, st) == cudaSuccess) return cudaSuccess;
+      cudaGetLastError();
+    }
   }
-  if constexpr (EQ == EQ_EULER && CHAR) {
+  if constexpr (kLanes1D<EQ, CHAR, R>) {
     if (ts.lanes == 4) {
       const int w = ts.width ? ts.width : 128;
       if (w == 32) return coop_launch<EQ, CHAR, R, 32, true>(A, nsteps, (nx + 5) / 6, st);
@@ -442,12 +469,15 @@ static size_t local1d_t() {
   size_t m = 0;
   if (!local_max(&m, stage1d_kernel<EQ, CHAR, R, 128>, stage1d_kernel<EQ, CHAR, R, 32>,
                  step1d_coop_kernel<EQ, CHAR, R, 128, false>,
-                 step1d_coop_kernel<EQ, CHAR, R, 32, false>,
-                 step1d_cluster_kernel<EQ, CHAR, R, false>))
+                 step1d_coop_kernel<EQ, CHAR, R, 32, false>))
     return 0;
-  if constexpr (EQ == EQ_EULER && CHAR) {
-    if (!local_max(&m, stage1d_fields_kernel<R, 32>, stage1d_fields_kernel<R, 64>,
-                   stage1d_fields_kernel<R, 128>, step1d_coop_kernel<EQ, CHAR, R, 32, true>,
+  if constexpr (sizeof(R) == sizeof(float)) {
+    if (!local_max(&m, step1d_cluster_kernel<EQ, CHAR, R, false>)) return 0;
+  }
+  if constexpr (kLanes1D<EQ, CHAR, R>) {
+    if (!local_max(&m, stage1d_lanes_kernel<EQ, CHAR, R, 32>, stage1d_lanes_kernel<EQ, CHAR, R, 64>,
+                   stage1d_lanes_kernel<EQ, CHAR, R, 128>,
+                   step1d_coop_kernel<EQ, CHAR, R, 32, true>,
                    step1d_coop_kernel<EQ, CHAR, R, 64, true>,
                    step1d_coop_kernel<EQ, CHAR, R, 128, true>,
                    step1d_cluster_kernel<EQ, CHAR, R, true>))

@@ -196,8 +196,7 @@ __device__ __forceinline__ void stage1d_item_io(const KProblem& P, const IO& io,
     }
   }
   // block max -> one atomic per block
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+  wmax = warp_max_nonneg(wmax);
   if ((t & 31) == 0) red[t >> 5] = wmax;
   __syncthreads();
   if (t == 0) {
@@ -207,12 +206,6 @@ __device__ __forceinline__ void stage1d_item_io(const KProblem& P, const IO& io,
     io.raise_alpha(m);
   }
   __syncthreads();  // the block may start another item in the same shared memory
-}
-
-template <int EQ, bool CHAR, typename R, int BW>
-__device__ __forceinline__ void stage1d_item(const KProblem& P, const KStage& S, int blk) {
-  const Global1D io{S, P.nx};
-  stage1d_item_io<EQ, CHAR, R, BW>(P, io, blk);
 }
 
 // One lane per characteristic field (1D Euler with the characteristic decomposition): the
@@ -342,8 +335,7 @@ __device__ __forceinline__ void stage1d_fields_item_io(const KProblem& P, const 
     io.nonphysical();
     wmax = 0.0;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+  wmax = warp_max_nonneg(wmax);
   if ((t & 31) == 0) red[t >> 5] = wmax;
   __syncthreads();
   if (t == 0) {
@@ -353,12 +345,6 @@ __device__ __forceinline__ void stage1d_fields_item_io(const KProblem& P, const 
     io.raise_alpha(m);
   }
   __syncthreads();  // the block may start another item in the same shared memory
-}
-
-template <typename R, int BW>
-__device__ __forceinline__ void stage1d_fields_item(const KProblem& P, const KStage& S, int blk) {
-  const Global1D io{S, P.nx};
-  stage1d_fields_item_io<R, BW>(P, io, blk);
 }
 
 }  // namespace hw

@@ -66,14 +66,14 @@ KProblem solve_kproblem(Solve* s);
 using namespace hw;
 
 // 1D: block width x threads per cell.  Candidates: 128- and 32-thread blocks of one thread per
-// cell, and for Euler with the characteristic decomposition 128-, 64- and 32-thread blocks of
-// one lane per characteristic field; each timed over eight stage launches (a 1D stage lasts
+// cell, and for FP64 solves and Euler with the characteristic decomposition 128-, 64- and
+// 32-thread blocks of four lanes per cell; each timed over eight stage launches (a 1D stage lasts
 // microseconds), the fastest kept.  *best_rows = block width, *best_bands = threads per cell.
 static int tune1d(const hweno_problem* p, Solve* s, cudaStream_t st, int* best_rows,
                   int* best_bands, double* best_ms) {
   const bool ch = p->equation == HWENO_EULER && p->characteristic;
   const int cand[5][2] = {{128, 1}, {32, 1}, {128, 4}, {64, 4}, {32, 4}};
-  const int ncand = ch ? 5 : 2;
+  const int ncand = ch || p->precision == HWENO_FP64 ? 5 : 2;
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
