@@ -140,7 +140,7 @@ static cudaError_t launch_batch1d_t(const BatchSolve* bs, BatchCtl* ctl, int k, 
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t init_batch_t(int* slots_out, size_t* local_out) {
-  constexpr int BW = batch_bw2d(sizeof(R) == 4);
+  constexpr int BW = kBatchBX;
   const size_t smem = smem_bytes2d<EQ, CHAR, R, BW>();
   auto kern = batch_stage_kernel<EQ, CHAR, R, BW>;
   static int slots = 0;
@@ -167,7 +167,7 @@ static cudaError_t init_batch_t(int* slots_out, size_t* local_out) {
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t launch_batch_t(const BatchSolve* bs, BatchCtl* ctl, int k, cudaStream_t st) {
-  constexpr int BW = batch_bw2d(sizeof(R) == 4);
+  constexpr int BW = kBatchBX;
   int slots = 0;
   cudaError_t e = init_batch_t<EQ, CHAR, R>(&slots, nullptr);
   if (e != cudaSuccess) return e;
@@ -264,8 +264,8 @@ int batch_slots(int cls) {
 
 void batch_geometry1d(int nx, int* blocks) { *blocks = (nx + (kBatchBW - 2) - 1) / (kBatchBW - 2); }
 
-void batch_geometry(int nx, int ny, int rows, bool mixed, int* bands, int* wout, int* chunks) {
-  split_bands(nx, default_bands(nx, batch_bw2d(mixed), false), bands, wout);
+void batch_geometry(int nx, int ny, int rows, int* bands, int* wout, int* chunks) {
+  split_bands(nx, default_bands(nx, kBatchBX, false), bands, wout);
   if (rows < 1) rows = 1;
   *chunks = (ny + rows - 1) / rows;
 }
@@ -274,11 +274,10 @@ int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots) 
   std::vector<int> bands(n), warps(n);
   for (int s = 0; s < n; ++s) {
     int wout, chunks;
-    batch_geometry(nx[s], ny[s], 1, mixed, &bands[s], &wout, &chunks);
+    batch_geometry(nx[s], ny[s], 1, &bands[s], &wout, &chunks);
     warps[s] = (wout + 2 + 31) / 32;
   }
-  return mixed ? batch_rows(bands.data(), ny, n, slots)
-               : batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX64, slots);
+  return batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX, slots, mixed);
 }
 
 }  // namespace hw

@@ -7,15 +7,13 @@
 
 namespace hw {
 
-// Block width of the batched stage kernels: the FP32-bulk and 1D classes 128 threads (the
-// FP32-bulk class's 192-thread blocks, faster for a solve alone, have not been measured here),
-// the 2D FP64 classes tiles of 64 columns x 3 rows (against one row at a time in 128-thread
-// blocks, which hold only four warps per SM: a batch of eight solves of 200 x 184 to 284 x 261
-// cells, one step, 9.00 -> 7.58 ms; a served mix of six grids of 128^2 to 352^2 cells in both
-// precisions, 114 -> 95.5 ms).
+// Block width of the batched stage kernels: the 1D classes 128 threads, the 2D classes tiles of 64
+// columns x 3 rows (against one row at a time in 128-thread blocks, which hold only four warps
+// per SM in FP64: a batch of eight FP64 solves of 200 x 184 to 284 x 261 cells, one step, 9.00 ->
+// 7.58 ms; a served mix of six grids of 128^2 to 352^2 cells, a third of them FP32-bulk, 114 ->
+// 95.5 ms with the FP64 classes in tiles).
 constexpr int kBatchBW = 128;
-constexpr int kBatchBX64 = 64;
-constexpr int batch_bw2d(bool mixed) { return mixed ? kBatchBW : kBatchBX64; }
+constexpr int kBatchBX = 64;
 constexpr int kBatchClasses = 16;  // {2D, 1D} x {advection, Burgers, Euler comp.-wise,
                                    // Euler char.} x {FP64, mixed}
 
@@ -48,8 +46,8 @@ struct BatchDt {
 };
 
 int batch_class(int equation, int characteristic, int mixed, int dim = 2);
-// bands of at most batch_bw2d() - 2 columns and row chunks of `rows` rows
-void batch_geometry(int nx, int ny, int rows, bool mixed, int* bands, int* wout, int* chunks);
+// bands of at most kBatchBX - 2 columns and row chunks of `rows` rows
+void batch_geometry(int nx, int ny, int rows, int* bands, int* wout, int* chunks);
 // rows per item for the 2D solves of one class (n grids) on `slots` resident blocks
 int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots);
 void batch_geometry1d(int nx, int* blocks);

@@ -94,22 +94,28 @@ inline Geom2D geom2d(int nx, int ny, int bw, int slots, int rows_fixed, int band
   return g;
 }
 
-// ---- FP64 tiles: bx columns x tile_rows64(bx) rows of threads per block (stage2d_tile64.cuh),
+// ---- Tiles: FP64 bx columns x tile_rows64(bx) rows of threads per block (stage2d_tile64.cuh),
 // six or seven warps, so that one block fills an SM's FP64 unit.
 constexpr int tile_rows64(int bx) { return bx == 32 ? 7 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
+// The same for the FP32-bulk kernels: six warps per block, two blocks per SM (128 columns: four
+// warps, three blocks).
+constexpr int tile_rows32(int bx) { return bx == 32 ? 6 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
 
 // Time of a block in units of one row of one warp at the SM's full FP64 rate (16 clocks per warp
 // instruction): `warps` warps per row, `rows` output rows in `pieces` pieces, each with two ring
 // rows (0.46 of a row's work: the y pass without its volume sums); and at least 4.6 per step of
 // by rows, because a warp alone takes 64 clocks per FP64 instruction (and about 15 % more
 // for what its loads do not hide).
-inline double tile_time64(int warps, int by, int rows, int pieces) {
+// The FP32-bulk kernels have the same shape with 7 instead of 4.6 (a warp-row is 9.2 us of an SM at
+// 2048^2, a lone step 65 us).
+constexpr double kStep64 = 4.6, kStep32 = 7.0;
+inline double tile_time64(int warps, int by, int rows, int pieces, double step = kStep64) {
   const double work = (double)warps * (rows + 0.92 * pieces);
   const double steps = (double)((rows + 2 * pieces + by - 1) / by);
-  return work > 4.6 * steps ? work : 4.6 * steps;
+  return work > step * steps ? work : step * steps;
 }
 
-// The default tile of an FP64 grid: over the widths bx[0..n-1] (with slots[] resident blocks per
+// The default tile of a grid: over the widths bx[0..n-1] (with slots[] resident blocks per
 // GPU each, on `sms` SMs) and the chunk heights (or one segment per SM), the launch whose most
 // loaded SM is done first.  240^2: 32 x 7, 8 bands x 19 chunks of 13 rows (13.9, against 18.4 in
 // 96 x 2 tiles); 2048^2: 96 x 2, 22 bands in 152 segments of 297 band-rows (897, against 930 or
@@ -118,18 +124,19 @@ struct Tile64 {
   int bx;
   int rows;  // output rows per chunk; < -1: segments of -rows band-rows
 };
-inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* slots, int n) {
+inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* slots, int n,
+                             bool mixed = false) {
   Tile64 best{96, 0};
   double best_time = 1e300;
   for (int q = 0; q < n; ++q) {
-    const int by = tile_rows64(bx[q]);
+    const int by = mixed ? tile_rows32(bx[q]) : tile_rows64(bx[q]);
     int bands, wout;
     split_bands(nx, default_bands(nx, bx[q], false), &bands, &wout);
     const int warps = (wout + 2 + 31) / 32;
     auto consider = [&](long long blocks, int rows, int pieces, int encoded) {
       const long long per_sm = (blocks + sms - 1) / sms;
       const long long waves = (blocks + slots[q] - 1) / slots[q];
-      const double step = tile_time64(0, by, rows, pieces);   // the latency bound alone
+      const double step = tile_time64(0, by, rows, pieces, mixed ? kStep32 : kStep64);
       const double work = (double)warps * (rows + 0.92 * pieces) * (double)per_sm;
       const double time = work > step * (double)waves ? work : step * (double)waves;
       if (time < 0.995 * best_time) {
@@ -145,18 +152,19 @@ inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* 
       consider((long long)bands * ((ny + r - 1) / r), r, 1, r);
     }
     const long long total = (long long)bands * ny;
-    const long long seg = (total + sms - 1) / sms;
-    if (bands <= sms && seg > 1)
+    const int parts = mixed ? slots[q] : sms;  // one FP64 block fills an SM, two FP32-bulk ones
+    const long long seg = (total + parts - 1) / parts;
+    if (bands <= parts && seg > 1)
       consider((total + seg - 1) / seg, (int)seg, (int)(1 + (seg - 1 + ny - 1) / ny), -(int)seg);
   }
   return best;
 }
 
-// Rows per item of a batched FP64 class in tiles of bx columns (bands[s] bands of warps[s] warps
+// Rows per item of a batched 2D class in tiles of bx columns (bands[s] bands of warps[s] warps
 // per row, ny[s] rows), whose persistent launch has `slots` resident blocks: the rows of least
 // waves x item time, the smallest (the most items) among equals.
 inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n, int bx,
-                        int slots) {
+                        int slots, bool mixed = false) {
   if (n <= 0 || slots <= 0) return 32;
   int nymax = 1;
   for (int s = 0; s < n; ++s) nymax = ny[s] > nymax ? ny[s] : nymax;
@@ -167,7 +175,9 @@ inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n
     double time = 0.0;
     for (int s = 0; s < n; ++s) {
       items += (long long)bands[s] * ((ny[s] + r - 1) / r);
-      const double t = tile_time64(warps[s], tile_rows64(bx), r < ny[s] ? r : ny[s], 1);
+      const double t =
+          tile_time64(warps[s], mixed ? tile_rows32(bx) : tile_rows64(bx), r < ny[s] ? r : ny[s],
+                      1, mixed ? kStep32 : kStep64);
       time = t > time ? t : time;
     }
     const double cost = (double)((items + slots - 1) / slots) * time;

@@ -189,7 +189,7 @@ static int rebuild_lists(Server* S, cudaStream_t st, unsigned* classes) {
     B.mixed = p->precision == HWENO_MIXED32;
     if (p->dim == 2) {
       B.rows = rows_of[cls];
-      batch_geometry(p->nx, p->ny, B.rows, B.mixed != 0, &B.bands, &B.wout, &B.chunks);
+      batch_geometry(p->nx, p->ny, B.rows, &B.bands, &B.wout, &B.chunks);
     } else {
       batch_geometry1d(p->nx, &B.bands);
       B.wout = kBatchBW - 2;

@@ -94,9 +94,9 @@ cudaError_t launch2d_width(int eq, bool characteristic, bool mixed, const KProbl
                            const KStage& S, TileShape t, cudaStream_t st);
 template <int BW>
 cudaError_t prepare2d_width(size_t* max_local);
-// resident blocks per GPU of the class's FP64 kernel in tiles BW columns wide
+// resident blocks per GPU of the class's kernel in tiles BW columns wide
 template <int BW>
-cudaError_t slots64_width(int eq, bool characteristic, int* slots);
+cudaError_t slots_width(int eq, bool characteristic, bool mixed, int* slots);
 #define HW_STAGE2D_DECLARE(BW)                                                                \
   template <>                                                                                 \
   cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool mixed, const KProblem& P,  \
@@ -104,7 +104,7 @@ cudaError_t slots64_width(int eq, bool characteristic, int* slots);
   template <>                                                                                 \
   cudaError_t prepare2d_width<BW>(size_t* max_local);                                         \
   template <>                                                                                 \
-  cudaError_t slots64_width<BW>(int eq, bool characteristic, int* slots);
+  cudaError_t slots_width<BW>(int eq, bool characteristic, bool mixed, int* slots);
 HW_STAGE2D_DECLARE(32)
 HW_STAGE2D_DECLARE(128)
 HW_STAGE2D_DECLARE(96)
@@ -112,39 +112,22 @@ HW_STAGE2D_DECLARE(64)
 HW_STAGE2D_DECLARE(192)
 #undef HW_STAGE2D_DECLARE
 
-// the FP64 classes of one width
-#define HW_STAGE2D_SLOTS64(BW)                                                                \
+#define HW_STAGE2D_SLOTS(BW)                                                                  \
   template <>                                                                                 \
-  cudaError_t slots64_width<BW>(int eq, bool characteristic, int* slots) {                    \
-    if (eq == EQ_ADV) return init2d_t<EQ_ADV, false, double, BW>(slots, nullptr);             \
-    if (eq == EQ_BURG) return init2d_t<EQ_BURG, false, double, BW>(slots, nullptr);           \
-    if (characteristic) return init2d_t<EQ_EULER, true, double, BW>(slots, nullptr);          \
-    return init2d_t<EQ_EULER, false, double, BW>(slots, nullptr);                             \
-  }
-#define HW_STAGE2D_WIDTH64(BW)                                                                \
-  HW_STAGE2D_SLOTS64(BW)                                                                      \
-  template <>                                                                                 \
-  cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool, const KProblem& P,        \
-                                 const KStage& S, TileShape t, cudaStream_t st) {             \
-    if (eq == EQ_ADV) return launch2d_w<EQ_ADV, false, double, BW>(P, S, t, st);              \
-    if (eq == EQ_BURG) return launch2d_w<EQ_BURG, false, double, BW>(P, S, t, st);            \
-    if (characteristic) return launch2d_w<EQ_EULER, true, double, BW>(P, S, t, st);           \
-    return launch2d_w<EQ_EULER, false, double, BW>(P, S, t, st);                              \
-  }                                                                                           \
-  template <>                                                                                 \
-  cudaError_t prepare2d_width<BW>(size_t* max_local) {                                        \
-    size_t m = 0, l = 0;                                                                      \
-    cudaError_t e = init2d_t<EQ_ADV, false, double, BW>(nullptr, &m);                         \
-    if (e == cudaSuccess && (e = init2d_t<EQ_BURG, false, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;   \
-    if (e == cudaSuccess && (e = init2d_t<EQ_EULER, false, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;  \
-    if (e == cudaSuccess && (e = init2d_t<EQ_EULER, true, double, BW>(nullptr, &l)) == cudaSuccess) m = l > m ? l : m;   \
-    if (max_local) *max_local = m;                                                            \
-    return e;                                                                                 \
+  cudaError_t slots_width<BW>(int eq, bool characteristic, bool mixed, int* slots) {          \
+    if (eq == EQ_ADV) return mixed ? init2d_t<EQ_ADV, false, float, BW>(slots, nullptr)       \
+                                   : init2d_t<EQ_ADV, false, double, BW>(slots, nullptr);     \
+    if (eq == EQ_BURG) return mixed ? init2d_t<EQ_BURG, false, float, BW>(slots, nullptr)     \
+                                    : init2d_t<EQ_BURG, false, double, BW>(slots, nullptr);   \
+    if (characteristic) return mixed ? init2d_t<EQ_EULER, true, float, BW>(slots, nullptr)    \
+                                     : init2d_t<EQ_EULER, true, double, BW>(slots, nullptr);  \
+    return mixed ? init2d_t<EQ_EULER, false, float, BW>(slots, nullptr)                       \
+                 : init2d_t<EQ_EULER, false, double, BW>(slots, nullptr);                     \
   }
 
 // every class of one width
 #define HW_STAGE2D_WIDTH(BW)                                                                  \
-  HW_STAGE2D_SLOTS64(BW)                                                                      \
+  HW_STAGE2D_SLOTS(BW)                                                                        \
   template <>                                                                                 \
   cudaError_t launch2d_width<BW>(int eq, bool characteristic, bool mixed, const KProblem& P,  \
                                  const KStage& S, TileShape t, cudaStream_t st) {             \

@@ -18,21 +18,19 @@
 
 namespace hw {
 
-
-// Threads of a block: bands of at most BW - 2 columns, one row at a time in the FP32-bulk
-// kernels, tile_rows64(BW) rows at once in the FP64 ones.
-template <int BW>
-constexpr int kTileRows64 = tile_rows64(BW);
+// Tile of a block: bands of at most BW - 2 columns, kTileRows rows at once (geometry.h).
 template <typename R, int BW>
-constexpr int kThreads2D = sizeof(R) == sizeof(double) ? BW * kTileRows64<BW> : BW;
+constexpr int kTileRows = sizeof(R) == sizeof(double) ? tile_rows64(BW) : tile_rows32(BW);
+template <typename R, int BW>
+constexpr int kThreads2D = BW * kTileRows<R, BW>;
 
 // Resident blocks per SM the 2D stage kernels are compiled for: the FP64 Euler kernels take the
 // register file and the shared memory with one block (two of 128 threads would not fit), the
-// scalar FP64 ones two; the FP32-bulk kernels twelve warps (at most 168 registers per thread: two
-// 192-thread, three 128-thread, four 96-thread or six 64-thread blocks), which hides more of
-// the FP64 latency of their weight evaluation.
+// scalar FP64 ones two; the FP32-bulk kernels twelve warps (at most 168 registers per thread),
+// which hides more of the FP64 latency of their weight evaluation.
 template <int EQ, typename R, int BW>
-constexpr int kMinBlocks2D = sizeof(R) == sizeof(double) ? (EQ == EQ_EULER ? 1 : 2) : 384 / BW;
+constexpr int kMinBlocks2D =
+    sizeof(R) == sizeof(double) ? (EQ == EQ_EULER ? 1 : 2) : 384 / kThreads2D<R, BW>;
 
 // Gauss weights on [-1/2, 1/2] (sum 1) and nodes
 #define GW0 (5.0 / 18.0)
@@ -76,78 +74,105 @@ template <int EQ, bool CHAR, typename R, int BW>
 constexpr size_t smem_bytes2d() {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
   if constexpr (sizeof(R) == sizeof(double))
-    return smem_bytes_tile64<EQ, CHAR, BW, kTileRows64<BW>>();
-  return sizeof(R) * 3 * NC * 3 * (BW + 2) + sizeof(R) * NC * 3 * 2 * BW +
-         sizeof(R) * 2 * 3 * NC * BW;
+    return smem_bytes_tile64<EQ, CHAR, BW, kTileRows<R, BW>>();
+  constexpr int BY = kTileRows<R, BW>;
+  return sizeof(R) * ((BY + 2) * 3 * NC * (BW + 2) + (6 + 2) * NC * BW * BY +
+                      6 * NC * BW * (BY + 1));
 }
 
-template <int EQ, bool CHAR, typename R, int BW>
+template <int EQ, bool CHAR, typename R, int BX, int BY>
 __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KStage& S, int band,
                                                    int j0, int j1, int wout, double* smem,
-                                                   double (*red)[BW / 32]) {
+                                                   double (*red)[BX * BY / 32]) {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;
   constexpr int NM = 3;
-  constexpr int NA = NC * NM;
-  constexpr int WC = BW + 2;  // window columns: global columns i0-2 .. i0+BW-1
-  // rows r-1, r, r+1 of the stage input for the reconstruction of row r, in slots r mod 3
-  // (row r+2 is loaded into the slot of row r-1 once every thread is done with it)
-  R* win = reinterpret_cast<R*>(smem);                  // [3 rows][NA][WC]
-  // x-face exchange, [NC][3][2][BW]: the left trace u and its flux f of every thread's cell;
-  // the face flux at the left face of thread x's cell then overwrites the u slot x (its only
-  // reader, thread x - 1, has read it by then)
-  R* trL = win + 3 * NA * WC;
-  auto fhx = [&](int cg, int x) -> R& { return trL[(cg * 2 + 0) * BW + x]; };
-  // top traces of (i, j-1) and g of them, carried to row j: [2][3][NC][BW] (each thread reads
-  // only its own column)
-  R* car = trL + NC * 3 * 2 * BW;
-  auto prevT = [&](int g, int c) -> R& { return car[((0 * 3 + g) * NC + c) * BW + threadIdx.x]; };
-  auto prevTg = [&](int g, int c) -> R& { return car[((1 * 3 + g) * NC + c) * BW + threadIdx.x]; };
+  constexpr int NA = NC * NM, T = BX * BY, NR = BY + 2;
+  constexpr int WC = BX + 2;  // window columns: global columns i0-2 .. i0+BX-1
+  const int t = threadIdx.x;
+  const int tx = t % BX, ty = t / BX;  // ty is uniform over a warp
+  // rows of the stage input for the reconstruction of the tile's rows, row r in slot
+  // (r - j0 + 2) mod NR
+  R* win = reinterpret_cast<R*>(smem);                  // [NR][NA][WC]
+  // x-face exchange of the thread's row, [NC][3][2][BX]: the left trace u and its flux f of every
+  // thread's cell; the face flux at the left face of thread x's cell then overwrites the u
+  // slot x (its only reader, thread x - 1, has read it by then)
+  R* trL = win + NR * NA * WC + ty * NC * 3 * 2 * BX;
+  auto fhx = [&](int cg, int x) -> R& { return trL[(cg * 2 + 0) * BX + x]; };
+  // the rows' top traces and g of them, [BY + 1][2][3][NC][BX] (the tile's last row alternates
+  // between two slots, as it is read a step later)
+  R* car = win + NR * NA * WC + NC * 3 * 2 * T;
+  // Gauss moments of the face below each row, [2 NC][T]
+  R* fm = car + (BY + 1) * 6 * NC * BX;
 
   const int nx = P.nx, ny = P.ny;
   const size_t plane = (size_t)nx * ny;
-  const int t = threadIdx.x;
-  const int i0 = band * wout;   // wout <= BW - 2 output columns per band
-  const int i = i0 - 1 + t;
-  const bool need = (t <= wout + 1) && (i <= nx);
-  const bool outc = (t >= 1 && t <= wout && i < nx);
+  const int i0 = band * wout;   // wout <= BX - 2 output columns per band
+  const int i = i0 - 1 + tx;
+  const bool lane = (tx <= wout + 1) && (i <= nx);
+  const bool outc = (tx >= 1 && tx <= wout && i < nx);
   const R a1 = (R)S.alpha_in[0], a2 = (R)S.alpha_in[1];
   const double dt = *S.dt;
   const R idx = kconst<R>(P.inv_dx, P.inv_dxf), idy = kconst<R>(P.inv_dy, P.inv_dyf);
   const R s15 = R(HW_S15);
 
+  // window column tx of a row is loaded by thread tx of a row's threads, the two last columns by
+  // threads 0 .. 2 NA - 1
+  int fx0, fx1;
+  const int ii0 = bc_map(i0 - 2 + tx, nx, P.bc[0], P.bc[1], fx0);
+  const int ii1 = bc_map(i0 - 2 + BX + tx / NA, nx, P.bc[0], P.bc[1], fx1);
   auto load_row = [&](int r) {
     int fy;
     const int rr = bc_map(r, ny, P.bc[2], P.bc[3], fy);
-    R* dst = win + ((r + 3) % 3) * NA * WC;  // r >= -2
-    for (int q = t; q < NA * WC; q += BW) {
-      const int a = q / WC, col = q - a * WC;
-      int fx;
-      const int ii = bc_map(i0 - 2 + col, nx, P.bc[0], P.bc[1], fx);
-      double val = S.Uin[(size_t)a * plane + (size_t)rr * nx + ii];
-      if (fx | fy) val *= mirror_sign<EQ, 2>(a / NM, a % NM, fx, fy);
-      dst[a * WC + col] = from_f64<R>(val);
+    R* dst = win + ((r - j0 + 2) % NR) * NA * WC;  // r >= j0 - 2
+    const double* src = S.Uin + (size_t)rr * nx;
+    double v[NA], v1 = 0.0;
+    const int a1_ = tx % NA;
+#pragma unroll
+    for (int a = 0; a < NA; ++a) v[a] = src[(size_t)a * plane + ii0];
+    if (tx < 2 * NA) v1 = src[(size_t)a1_ * plane + ii1];
+    if (fx0 | fy) {
+#pragma unroll
+      for (int a = 0; a < NA; ++a) v[a] *= mirror_sign<EQ, 2>(a / NM, a % NM, fx0, fy);
     }
+    if (tx < 2 * NA && (fx1 | fy)) v1 *= mirror_sign<EQ, 2>(a1_ / NM, a1_ % NM, fx1, fy);
+#pragma unroll
+    for (int a = 0; a < NA; ++a) dst[a * WC + tx] = from_f64<R>(v[a]);
+    if (tx < 2 * NA) dst[a1_ * WC + BX + tx / NA] = from_f64<R>(v1);
   };
 #pragma unroll 1
-  for (int r = j0 - 2; r <= j0; ++r) load_row(r);
+  for (int r = j0 - 2 + ty; r <= j0 - 1 + BY && r <= j1 + 1; r += BY) load_row(r);
   __syncthreads();
+  // the threads of a row wait for each other (named barrier of the row; a warp on its own)
+  auto row_sync = [&]() {
+    if constexpr (BX == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + ty), "n"(BX) : "memory");
+  };
 
-  // state carried from row j-1 to row j
-  R pend[NC][3];                   // F^1..F^3 of (i, j-1) without its top face
-  R pvh[NC], pwh[NC];              // v-hat, w-hat of (i, j-1)
+  // the row waiting for the face above it (used by the threads of the tile's last row)
+  R pend[NC][3];
+  R pvh[NC], pwh[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) pend[c][0] = pend[c][1] = pend[c][2] = pvh[c] = pwh[c] = R(0);
   double wmax0 = 0.0, wmax1 = 0.0;
   bool fast_weights = true;        // cleared where the direct-formula weights were needed
 
 #pragma unroll 1
-  for (int j = j0 - 1; j <= j1; ++j) {
-    const R* wm = win + ((j + 2) % 3) * NA * WC;  // j >= -1
-    const R* w0 = win + ((j + 3) % 3) * NA * WC;
-    const R* wp = win + ((j + 4) % 3) * NA * WC;
+  for (int step = 0;; ++step) {
+    const int jb = j0 - 1 + step * BY;
+    if (jb > j1) break;  // uniform over the block
+    const int j = jb + ty;
+    const bool need = lane && j <= j1;
+    const int slot = step * BY + ty;  // of the row below
+    const R* wm = win + (slot % NR) * NA * WC;
+    const R* w0 = win + ((slot + 1) % NR) * NA * WC;
+    const R* wp = win + ((slot + 2) % NR) * NA * WC;
     auto Wv = [&](int a, int k) -> R {   // moment array a of stencil cell k (0..8)
       const R* rowp = (k < 3) ? wm : (k < 6 ? w0 : wp);
-      return rowp[a * WC + t + (k % 3)];
+      return rowp[a * WC + tx + (k % 3)];
     };
-    const bool xrow = (j >= j0 && j < j1);
+    const bool xrow = (j >= j0 && j < j1);  // uniform over a row's threads
+    R* cmine = car + (ty < BY - 1 ? ty : BY - 1 + (step & 1)) * 6 * NC * BX + tx;
+    const R* cbelow = car + (ty > 0 ? ty - 1 : BY - 1 + ((step + 1) & 1)) * 6 * NC * BX + tx;
 
     R xl[3][NC], xr[3][NC], volf[NC], vh[NC];
     R yb[3][NC], yt[3][NC], volg[NC], wh[NC];
@@ -156,7 +181,7 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
     for (int c = 0; c < NC; ++c) rx[c][0] = rx[c][1] = rx[c][2] = R(0);
 
     // x faces of row j (output rows only): traces through shared memory, one flux per face;
-    // called by every thread of the block (it synchronises)
+    // called by every thread of the row (they synchronise)
     auto xfaces = [&]() {
       R fl[3][NC], fr[3][NC];
       if (need) {
@@ -166,30 +191,30 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
           flux_dir<EQ, R>(P, 0, xr[g], fr[g]);
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            trL[((c * 3 + g) * 2 + 0) * BW + t] = xl[g][c];
-            trL[((c * 3 + g) * 2 + 1) * BW + t] = fl[g][c];
+            trL[((c * 3 + g) * 2 + 0) * BX + tx] = xl[g][c];
+            trL[((c * 3 + g) * 2 + 1) * BX + tx] = fl[g][c];
           }
         }
       }
-      __syncthreads();
-      if (need && t <= wout && i < nx) {
+      row_sync();
+      if (need && tx <= wout && i < nx) {
 #pragma unroll
         for (int g = 0; g < 3; ++g)
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            const R uR = trL[((c * 3 + g) * 2 + 0) * BW + t + 1];
-            const R fR = trL[((c * 3 + g) * 2 + 1) * BW + t + 1];
+            const R uR = trL[((c * 3 + g) * 2 + 0) * BX + tx + 1];
+            const R fR = trL[((c * 3 + g) * 2 + 1) * BX + tx + 1];
             // twice the LF flux (Eq. 2.4 without its factor 1/2, folded into the weights)
-            fhx(c * 3 + g, t + 1) = fr[g][c] + fR - a1 * (uR - xr[g][c]);
+            fhx(c * 3 + g, tx + 1) = fr[g][c] + fR - a1 * (uR - xr[g][c]);
           }
       }
-      __syncthreads();
+      row_sync();
       if (outc) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          const R L0 = fhx(c * 3 + 0, t), L1 = fhx(c * 3 + 1, t), L2 = fhx(c * 3 + 2, t);
-          const R R0 = fhx(c * 3 + 0, t + 1), R1 = fhx(c * 3 + 1, t + 1),
-                  R2 = fhx(c * 3 + 2, t + 1);
+          const R L0 = fhx(c * 3 + 0, tx), L1 = fhx(c * 3 + 1, tx), L2 = fhx(c * 3 + 2, tx);
+          const R R0 = fhx(c * 3 + 0, tx + 1), R1 = fhx(c * 3 + 1, tx + 1),
+                  R2 = fhx(c * 3 + 2, tx + 1);
           const R sdiff = R(0.5 * GW0) * ((R0 - L0) + (R2 - L2)) + R(0.5 * GW1) * (R1 - L1);
           const R ssum = R(0.5 * GW0) * ((L0 + R0) + (L2 + R2)) + R(0.5 * GW1) * (L1 + R1);
           const R smom = R(0.5 * GW0) * s15 * ((R2 - L2) - (R0 - L0));
@@ -374,12 +399,23 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
       if (xrow) xfaces();
     }
 
-    // y face j-1/2 between (i, j-1) (top traces kept) and (i, j) (bottom traces): Eq. 2.16
+    // y face j-1/2 between (i, j-1) and (i, j): Eq. 2.16
     R ybg[3][NC];
     if (need) {
 #pragma unroll
       for (int g = 0; g < 3; ++g) flux_dir<EQ, R>(P, 1, yb[g], ybg[g]);
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        R tg[NC];
+        flux_dir<EQ, R>(P, 1, yt[g], tg);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          cmine[(g * NC + c) * BX] = yt[g][c];
+          cmine[((3 + g) * NC + c) * BX] = tg[c];
+        }
+      }
     }
+    __syncthreads();  // the step's traces are in place and nothing reads the window any more
     R rhs[NC][3];
 #pragma unroll
     for (int c = 0; c < NC; ++c) rhs[c][0] = rhs[c][1] = rhs[c][2] = R(0);
@@ -389,104 +425,103 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
       for (int g = 0; g < 3; ++g)
 #pragma unroll
         for (int c = 0; c < NC; ++c)
-          gh[g][c] = prevTg(g, c) + ybg[g][c] - a2 * (yb[g][c] - prevT(g, c));  // 2 x LF flux
+          gh[g][c] = cbelow[((3 + g) * NC + c) * BX] + ybg[g][c] -
+                     a2 * (yb[g][c] - cbelow[(g * NC + c) * BX]);  // 2 x LF flux
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const R sw = R(0.5 * GW0) * (gh[0][c] + gh[2][c]) + R(0.5 * GW1) * gh[1][c];
         const R sm = R(0.5 * GW0) * s15 * (gh[2][c] - gh[0][c]);
-        // top face of (i, j-1): F1 -= sum/dy, F2 -= sum xi/dy, F3 -= sum/(2 dy)
-        pend[c][0] -= sw * idy;
-        pend[c][1] -= sm * idy;
-        pend[c][2] -= R(0.5) * sw * idy;
+        fm[(2 * c) * T + t] = sw;
+        fm[(2 * c + 1) * T + t] = sm;
         // bottom face of (i, j): F1 += sum/dy, F2 += sum xi/dy, F3 -= sum/(2 dy)
-        rhs[c][0] = sw * idy;
-        rhs[c][1] = sm * idy;
-        rhs[c][2] = -R(0.5) * sw * idy;
-      }
-      // stage update of (i, j-1): Eq. 2.13
-      if (outc && j - 1 >= j0) {
-        const size_t q = (size_t)(j - 1) * nx + i;
-        double outv[NC * NM];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const double own_u = (sizeof(R) == sizeof(double))
-                                   ? (double)wm[(c * NM) * WC + t + 1]
-                                   : S.Uin[(size_t)(c * NM) * plane + q];
-          const double own[3] = {own_u, to_f64(pvh[c]), to_f64(pwh[c])};
-#pragma unroll
-          for (int m = 0; m < 3; ++m) {
-            const size_t qa = (size_t)(c * NM + m) * plane + q;
-            double base;
-            if (S.k == 1) {
-              base = own[m];
-              if (m > 0) S.Vh[(size_t)(c * 2 + m - 1) * plane + q] = own[m];
-            } else {
-              base = (m == 0) ? S.Un[qa] : S.Vh[(size_t)(c * 2 + m - 1) * plane + q];
-            }
-            const double adv = fma(dt, to_f64(pend[c][m]), own[m]);
-            double o;
-            if (S.k == 1) o = adv;
-            else if (S.k == 2) o = fma(0.75, base, 0.25 * adv);
-            else o = fma(1.0 / 3.0, base, 2.0 / 3.0 * adv);
-            S.Uout[qa] = o;
-            outv[c * NM + m] = o;
-          }
-        }
-        double ua[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ua[c] = outv[c * NM];
-        bool bad = false;
-#pragma unroll
-        for (int q2 = 0; q2 < NC * NM; ++q2) bad |= !finite_bits(outv[q2]);
-        if constexpr (EQ == EQ_EULER) {
-          double s0, s1;
-          bad |= !euler_speeds<2>(P, ua, s0, s1);
-          if (!bad) {
-            wmax0 = fmax(wmax0, s0);
-            wmax1 = fmax(wmax1, s1);
-          }
-        } else {
-          wmax0 = fmax(wmax0, Phys<EQ, double>::speed(P, 0, ua));
-          wmax1 = fmax(wmax1, Phys<EQ, double>::speed(P, 1, ua));
-        }
-        if (bad) atomicOr(S.status, kStatusNonphysical);
+        rhs[c][0] = __fmul_rn(sw, idy);
+        rhs[c][1] = __fmul_rn(sm, idy);
+        rhs[c][2] = __fmul_rn(-R(0.5) * sw, idy);
       }
     }
-
     // the x-face and volume terms of (i, j)
     if (xrow && outc) {
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        rhs[c][0] += rx[c][0];
-        rhs[c][1] += rx[c][1];
-        rhs[c][2] += volg[c] * idy + rx[c][2];
+        rhs[c][0] = __fadd_rn(rhs[c][0], rx[c][0]);
+        rhs[c][1] = __fadd_rn(rhs[c][1], rx[c][1]);
+        rhs[c][2] = __fadd_rn(rhs[c][2], __fmaf_rn(volg[c], idy, rx[c][2]));
       }
     }
+    // the window's next BY rows, into the slots of the rows no longer needed
+    if (j + BY + 1 <= j1 + 1) load_row(j + BY + 1);
+    __syncthreads();
 
-    // carry row j to the next iteration
-    if (need) {
-#pragma unroll
-      for (int g = 0; g < 3; ++g) {
-        R tg[NC];
-        flux_dir<EQ, R>(P, 1, yt[g], tg);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          prevT(g, c) = yt[g][c];
-          prevTg(g, c) = tg[c];
-        }
-      }
+    // the row whose top face is now known: this thread's row j, or in the tile's last row the
+    // one it processed a step ago (row j takes its place)
+    const bool last = ty == BY - 1;
+    const int jc = last ? j - BY : j;
+    const R* face = fm + (last ? tx : t + BX);
+    if (last) {
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        pend[c][0] = rhs[c][0];
-        pend[c][1] = rhs[c][1];
-        pend[c][2] = rhs[c][2];
-        pvh[c] = vh[c];
-        pwh[c] = wh[c];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          const R x = rhs[c][m];
+          rhs[c][m] = pend[c][m];
+          pend[c][m] = x;
+        }
+        const R x = vh[c], y = wh[c];
+        vh[c] = pvh[c];
+        wh[c] = pwh[c];
+        pvh[c] = x;
+        pwh[c] = y;
       }
     }
-    __syncthreads();                       // every read of row j-1 is done
-    if (j + 2 <= j1 + 1) load_row(j + 2);  // into the slot of row j-1
-    __syncthreads();
+    if (outc && jc >= j0 && jc < j1) {
+      // its top face: F1 -= sum/dy, F2 -= sum xi/dy, F3 -= sum/(2 dy); then the update: Eq. 2.13
+      const size_t q = (size_t)jc * nx + i;
+      double outv[NC * NM];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const R sw = face[(2 * c) * T], sm = face[(2 * c + 1) * T];
+        rhs[c][0] = __fsub_rn(rhs[c][0], __fmul_rn(sw, idy));
+        rhs[c][1] = __fsub_rn(rhs[c][1], __fmul_rn(sm, idy));
+        rhs[c][2] = __fsub_rn(rhs[c][2], __fmul_rn(R(0.5) * sw, idy));
+        const double own[3] = {S.Uin[(size_t)(c * NM) * plane + q], to_f64(vh[c]), to_f64(wh[c])};
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          const size_t qa = (size_t)(c * NM + m) * plane + q;
+          double base;
+          if (S.k == 1) {
+            base = own[m];
+            if (m > 0) S.Vh[(size_t)(c * 2 + m - 1) * plane + q] = own[m];
+          } else {
+            base = (m == 0) ? S.Un[qa] : S.Vh[(size_t)(c * 2 + m - 1) * plane + q];
+          }
+          const double adv = fma(dt, to_f64(rhs[c][m]), own[m]);
+          double o;
+          if (S.k == 1) o = adv;
+          else if (S.k == 2) o = fma(0.75, base, 0.25 * adv);
+          else o = fma(1.0 / 3.0, base, 2.0 / 3.0 * adv);
+          S.Uout[qa] = o;
+          outv[c * NM + m] = o;
+        }
+      }
+      double ua[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) ua[c] = outv[c * NM];
+      bool bad = false;
+#pragma unroll
+      for (int q2 = 0; q2 < NC * NM; ++q2) bad |= !finite_bits(outv[q2]);
+      if constexpr (EQ == EQ_EULER) {
+        double s0, s1;
+        bad |= !euler_speeds<2>(P, ua, s0, s1);
+        if (!bad) {
+          wmax0 = fmax(wmax0, s0);
+          wmax1 = fmax(wmax1, s1);
+        }
+      } else {
+        wmax0 = fmax(wmax0, Phys<EQ, double>::speed(P, 0, ua));
+        wmax1 = fmax(wmax1, Phys<EQ, double>::speed(P, 1, ua));
+      }
+      if (bad) atomicOr(S.status, kStatusNonphysical);
+    }
   }
 
   // block maxima of the output wave speeds -> one atomic per block and direction
@@ -505,7 +540,7 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
     if (any_direct) atomicOr(S.status, kStatusDirectWeights);
     double m0 = red[0][0], m1 = red[1][0];
 #pragma unroll
-    for (int w = 1; w < BW / 32; ++w) {
+    for (int w = 1; w < T / 32; ++w) {
       m0 = fmax(m0, red[0][w]);
       m1 = fmax(m1, red[1][w]);
     }
@@ -521,9 +556,9 @@ __device__ __forceinline__ void stage2d_item(const KProblem& P, const KStage& S,
                                              int j0, int j1, int wout, double* smem,
                                              double (*red)[kThreads2D<R, BW> / 32]) {
   if constexpr (sizeof(R) == sizeof(double))
-    stage2d_tile64_item<EQ, CHAR, BW, kTileRows64<BW>>(P, S, band, j0, j1, wout, smem, red);
+    stage2d_tile64_item<EQ, CHAR, BW, kTileRows<R, BW>>(P, S, band, j0, j1, wout, smem, red);
   else
-    stage2d_mixed_item<EQ, CHAR, R, BW>(P, S, band, j0, j1, wout, smem, red);
+    stage2d_mixed_item<EQ, CHAR, R, BW, kTileRows<R, BW>>(P, S, band, j0, j1, wout, smem, red);
 }
 
 }  // namespace hw

@@ -1,9 +1,9 @@
-// stage2d_w32.cu -- the 32-column FP64 instantiations of the single-solve 2D stage kernel
+// stage2d_w32.cu -- the 32-column instantiations of the single-solve 2D stage kernel
 // (stage2d_impl.cuh), compiled apart from the other widths.
 #include "stage2d_impl.cuh"
 
 namespace hw {
 
-HW_STAGE2D_WIDTH64(32)
+HW_STAGE2D_WIDTH(32)
 
 }  // namespace hw

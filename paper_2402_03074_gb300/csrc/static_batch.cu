@@ -109,7 +109,7 @@ static bool g_static_ready[64];
 
 template <int EQ, bool CHAR, typename R>
 static cudaError_t static_class_setup(int* slots, size_t* local) {
-  constexpr int BW = batch_bw2d(sizeof(R) == 4);
+  constexpr int BW = kBatchBX;
   auto kern = static_batch_kernel<EQ, CHAR, R, BW>;
   const size_t smem = smem_bytes2d<EQ, CHAR, R, BW>();
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -129,7 +129,7 @@ static cudaError_t static_class_setup(int* slots, size_t* local) {
 
 template <int EQ, bool CHAR, typename R>
 static void static_launch(int slots, StaticScratch* ptr, int k, cudaStream_t st) {
-  constexpr int BW = batch_bw2d(sizeof(R) == 4);
+  constexpr int BW = kBatchBX;
   static_batch_kernel<EQ, CHAR, R, BW>
       <<<slots, kThreads2D<R, BW>, smem_bytes2d<EQ, CHAR, R, BW>(), st>>>(ptr, k);
 }
@@ -231,7 +231,7 @@ extern "C" int hweno_stage_batch_static(int n, const hweno_problem* problems, in
     it.dt = dt[s];
     it.status = status[s];
     it.rows = rows;
-    batch_geometry(nxs[s], nys[s], rows, mixed, &it.bands, &it.wout, &it.chunks);
+    batch_geometry(nxs[s], nys[s], rows, &it.bands, &it.wout, &it.chunks);
     it.item_base = items;
     items += it.bands * it.chunks;
   }
