@@ -270,6 +270,13 @@ void batch_geometry(int nx, int ny, int rows, int* bands, int* wout, int* chunks
   *chunks = (ny + rows - 1) / rows;
 }
 
+static int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
+
 int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots) {
   std::vector<int> bands(n), warps(n);
   for (int s = 0; s < n; ++s) {
@@ -277,7 +284,9 @@ int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots) 
     batch_geometry(nx[s], ny[s], 1, &bands[s], &wout, &chunks);
     warps[s] = (wout + 2 + 31) / 32;
   }
-  return batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX, slots, mixed);
+  const int sms = sm_count();
+  return batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX, slots,
+                      slots > sms ? slots / sms : 1, mixed);
 }
 
 }  // namespace hw

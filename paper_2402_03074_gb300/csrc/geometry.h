@@ -101,25 +101,28 @@ constexpr int tile_rows64(int bx) { return bx == 32 ? 7 : bx == 64 ? 3 : bx == 9
 // warps, three blocks).
 constexpr int tile_rows32(int bx) { return bx == 32 ? 6 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
 
-// Time of a block in units of one row of one warp at the SM's full FP64 rate (16 clocks per warp
-// instruction): `warps` warps per row, `rows` output rows in `pieces` pieces, each with two ring
-// rows (0.46 of a row's work: the y pass without its volume sums); and at least 4.6 per step of
-// by rows, because a warp alone takes 64 clocks per FP64 instruction (and about 15 % more
-// for what its loads do not hide).
-// The FP32-bulk kernels have the same shape with 7 instead of 4.6 (a warp-row is 9.2 us of an SM at
-// 2048^2, a lone step 65 us).
+// Time of `blocks` blocks sharing an SM, each sweeping a piece of `rows` output rows (and the two
+// ring rows, 0.46 of a row's work each: the y pass without its volume sums) by rows at a time, in
+// units of one row of one warp at the SM's full rate: a step takes the work of its rows
+// (`warps` warps each), but at least `step`, because a warp alone runs far below that rate (one FP64
+// instruction in 64 clocks against the SM's 16).  kStep64: 4.6 (40^2 Euler: 108 us per stage, a
+// warp-row 21 us of an SM at 2048^2); kStep32, the FP32-bulk kernels: 7 (65 us and 9.2 us).
 constexpr double kStep64 = 4.6, kStep32 = 7.0;
-inline double tile_time64(int warps, int by, int rows, int pieces, double step = kStep64) {
-  const double work = (double)warps * (rows + 0.92 * pieces);
-  const double steps = (double)((rows + 2 * pieces + by - 1) / by);
-  return work > step * steps ? work : step * steps;
+inline double tile_time64(int warps, int by, int rows, int blocks, double step) {
+  const int full = (rows + 2) / by, rest = (rows + 2) % by;
+  const double w = (double)warps * blocks;
+  // a last step of one row holds the upper ring row alone: half a step
+  const double last = rest == 1 ? 0.5 * step : rest ? (w * rest > step ? w * rest : step) : 0.0;
+  const double t = full * (w * by > step ? w * by : step) + last - 1.08 * w;
+  const double least = step * (full + (rest > 1 ? 1.0 : 0.5 * rest));
+  return t > least ? t : least;
 }
 
-// The default tile of a grid: over the widths bx[0..n-1] (with slots[] resident blocks per
-// GPU each, on `sms` SMs) and the chunk heights (or one segment per SM), the launch whose most
-// loaded SM is done first.  240^2: 32 x 7, 8 bands x 19 chunks of 13 rows (13.9, against 18.4 in
-// 96 x 2 tiles); 2048^2: 96 x 2, 22 bands in 152 segments of 297 band-rows (897, against 930 or
-// more in narrower bands, whose ring columns cost 3 and 7 % instead of 2 %).
+// The default tile of a grid: over the widths bx[0..n-1] (with slots[] resident blocks per GPU
+// each, on `sms` SMs) and the chunk heights (or one segment per resident block), the launch of
+// least time.  240^2 FP64: 32 x 7, 8 bands x 19 chunks of 13 rows (1.00 ms per three stages,
+// 1.06 in 64 x 3 tiles, 1.45 in rows of 192); 2048^2 FP64: 96 x 2, 22 bands in 152 segments of 297
+// band-rows (56.5 ms; 57.3 in 32 x 7, whose ring columns cost 7 % instead of 2 %).
 struct Tile64 {
   int bx;
   int rows;  // output rows per chunk; < -1: segments of -rows band-rows
@@ -128,43 +131,50 @@ inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* 
                              bool mixed = false) {
   Tile64 best{96, 0};
   double best_time = 1e300;
+  const double step = mixed ? kStep32 : kStep64;
   for (int q = 0; q < n; ++q) {
     const int by = mixed ? tile_rows32(bx[q]) : tile_rows64(bx[q]);
     int bands, wout;
     split_bands(nx, default_bands(nx, bx[q], false), &bands, &wout);
     const int warps = (wout + 2 + 31) / 32;
-    auto consider = [&](long long blocks, int rows, int pieces, int encoded) {
-      const long long per_sm = (blocks + sms - 1) / sms;
-      const long long waves = (blocks + slots[q] - 1) / slots[q];
-      const double step = tile_time64(0, by, rows, pieces, mixed ? kStep32 : kStep64);
-      const double work = (double)warps * (rows + 0.92 * pieces) * (double)per_sm;
-      const double time = work > step * (double)waves ? work : step * (double)waves;
+    const int per_sm = slots[q] > sms ? slots[q] / sms : 1;
+    // every wave and every further piece of a segment (`extra`) costs a window prologue, about 2.5
+    // units, the piece also its ring rows (1024^2 FP64: one wave of segments in two pieces 14.70 ms,
+    // three waves of 25-row chunks 14.98 ms)
+    constexpr double prologue = 2.5;
+    auto consider = [&](long long blocks, int rows, int extra, int encoded) {
+      const long long waves = blocks / slots[q], rest = blocks % slots[q];
+      double time = 0.0;
+      if (waves > 0) time += (double)waves * tile_time64(warps, by, rows, per_sm, step);
+      if (rest > 0)
+        time += tile_time64(warps, by, rows, (int)((rest + sms - 1) / sms), step);
+      time += (double)(waves + (rest > 0 ? 1 : 0)) * prologue +
+              extra * (prologue + 0.92 * warps * per_sm);
       if (time < 0.995 * best_time) {
         best_time = time;
         best = Tile64{bx[q], encoded};
       }
     };
-    for (int r = 1; r <= 16 && r <= ny; ++r) consider((long long)bands * ((ny + r - 1) / r), r, 1, r);
+    for (int r = 1; r <= 16 && r <= ny; ++r) consider((long long)bands * ((ny + r - 1) / r), r, 0, r);
     for (int m = 1; m <= 6; ++m) {
       int c = m * sms / bands;
       c = c < 1 ? 1 : (c > ny ? ny : c);
       const int r = (ny + c - 1) / c;
-      consider((long long)bands * ((ny + r - 1) / r), r, 1, r);
+      consider((long long)bands * ((ny + r - 1) / r), r, 0, r);
     }
     const long long total = (long long)bands * ny;
-    const int parts = mixed ? slots[q] : sms;  // one FP64 block fills an SM, two FP32-bulk ones
-    const long long seg = (total + parts - 1) / parts;
-    if (bands <= parts && seg > 1)
-      consider((total + seg - 1) / seg, (int)seg, (int)(1 + (seg - 1 + ny - 1) / ny), -(int)seg);
+    const long long seg = (total + slots[q] - 1) / slots[q];
+    if (bands <= slots[q] && seg > 1)
+      consider((total + seg - 1) / seg, (int)seg, (int)((seg - 1 + ny - 1) / ny), -(int)seg);
   }
   return best;
 }
 
 // Rows per item of a batched 2D class in tiles of bx columns (bands[s] bands of warps[s] warps
 // per row, ny[s] rows), whose persistent launch has `slots` resident blocks: the rows of least
-// waves x item time, the smallest (the most items) among equals.
+// waves x item time (per_sm blocks sharing an SM), the smallest (the most items) among equals.
 inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n, int bx,
-                        int slots, bool mixed = false) {
+                        int slots, int per_sm, bool mixed = false) {
   if (n <= 0 || slots <= 0) return 32;
   int nymax = 1;
   for (int s = 0; s < n; ++s) nymax = ny[s] > nymax ? ny[s] : nymax;
@@ -177,7 +187,7 @@ inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n
       items += (long long)bands[s] * ((ny[s] + r - 1) / r);
       const double t =
           tile_time64(warps[s], mixed ? tile_rows32(bx) : tile_rows64(bx), r < ny[s] ? r : ny[s],
-                      1, mixed ? kStep32 : kStep64);
+                      per_sm, mixed ? kStep32 : kStep64);
       time = t > time ? t : time;
     }
     const double cost = (double)((items + slots - 1) / slots) * time;

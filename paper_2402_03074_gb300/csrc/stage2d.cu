@@ -19,16 +19,15 @@ cudaError_t launch_stage2d(int eq, bool characteristic, bool mixed, const KProbl
   int w = t.width > 0 ? t.width : kDefaultWidth2D;
   if (w == kDefaultWidth2D && t.rows >= -1 && t.rows <= 0 && t.bands <= 0) {
     // the default: the tile width and chunk height of least time for the grid (geometry.h)
-    static const int bx[4] = {96, 64, 32, 192};
-    int slots[4], sms = 0, dev = 0;
-    cudaError_t e = slots_width<96>(eq, ch, mixed, &slots[0]);
+    static const int bx[3] = {32, 64, 96};
+    int slots[3], sms = 0, dev = 0;
+    cudaError_t e = slots_width<32>(eq, ch, mixed, &slots[0]);
     if (e == cudaSuccess) e = slots_width<64>(eq, ch, mixed, &slots[1]);
-    if (e == cudaSuccess) e = slots_width<32>(eq, ch, mixed, &slots[2]);
-    if (e == cudaSuccess) e = slots_width<192>(eq, ch, mixed, &slots[3]);
+    if (e == cudaSuccess) e = slots_width<96>(eq, ch, mixed, &slots[2]);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const Tile64 d = default_tile64(P.nx, P.ny, sms > 0 ? sms : 1, bx, slots, 4, mixed);
+    const Tile64 d = default_tile64(P.nx, P.ny, sms > 0 ? sms : 1, bx, slots, 3, mixed);
     w = d.bx;
     t.rows = d.rows;
   }
