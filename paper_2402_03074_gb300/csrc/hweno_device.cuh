@@ -380,66 +380,6 @@ __device__ __forceinline__ void coeffs2d(const R (&u)[9], const R (&v)[4], const
   c[14] = R(-5.0 / 8.0) * vv + R(5.0 / 4.0) * u5 + R(15.0 / 4.0) * Wd;
 }
 
-// Steps 2-3 inputs: the smoothness indicators of Eq. 2.20 (double) of p_0 (coefficients c)
-// and of the linear polynomials on S_1 = {2,4,5}, S_2 = {2,5,6}, S_3 = {4,5,8}, S_4 = {5,6,8}
-// (slopes u5 - u4, u6 - u5, u5 - u2, u8 - u5), and u_ave of Eq. 2.22.
-template <typename R>
-__device__ __forceinline__ void beta2d(const R (&c)[15], const R (&u)[9], double (&beta)[5],
-                                       double& uave) {
-  double d[15];
-#pragma unroll
-  for (int n = 0; n < 15; ++n) d[n] = to_f64(c[n]);
-  double s, t;
-  t = fma(0.5, d[6], d[1]);
-  s = t * t;
-  t = fma(1.0 / 6.0, d[8], d[1]);
-  s = fma(t, t, s);
-  t = fma(1.0 / 6.0, d[7], d[2]);
-  s = fma(t, t, s);
-  t = fma(0.5, d[9], d[2]);
-  s = fma(t, t, s);
-  double b = 0.5 * s;
-  t = fma(63.0 / 65.0, d[10], d[3]);
-  s = t * t;
-  t = fma(1.0 / 6.0, d[12], d[3]);
-  s = fma(t, t, s);
-  t = fma(1.0 / 6.0, d[12], d[5]);
-  s = fma(t, t, s);
-  t = fma(63.0 / 65.0, d[14], d[5]);
-  s = fma(t, t, s);
-  b = fma(13.0 / 6.0, s, b);
-  t = fma(17.0 / 35.0, d[11], d[4]);
-  s = t * t;
-  t = fma(17.0 / 35.0, d[13], d[4]);
-  s = fma(t, t, s);
-  b = fma(7.0 / 12.0, s, b);
-  t = fma(5.0 / 9357.0, d[8], d[6]);
-  b = fma(3119.0 / 80.0 * t, t, b);
-  t = fma(15.0 / 3379.0, d[9], d[7]);
-  b = fma(3379.0 / 720.0 * t, t, b);
-  b = fma(2634769.0 / 561420.0 * d[8], d[8], b);
-  b = fma(2634769.0 / 67580.0 * d[9], d[9], b);
-  t = fma(3185.0 / 11353166.0, d[12], d[10]);
-  b = fma(5676583.0 / 9100.0 * t, t, b);
-  t = fma(1155.0 / 709573.0, d[13], d[11]);
-  b = fma(709573.0 / 16800.0 * t, t, b);
-  t = fma(2145748374.0 / 230094013357.0, d[14], d[12]);
-  b = fma(230094013357.0 / 12261419280.0 * t, t, b);
-  b = fma(31468281769.0 / 745051650.0 * d[13], d[13], b);
-  b = fma(25118160529227568.0 / 40266452337475.0 * d[14], d[14], b);
-  beta[0] = b;
-  const double el = to_f64(u[4] - u[3]), er = to_f64(u[5] - u[4]), eb = to_f64(u[4] - u[1]),
-               et = to_f64(u[7] - u[4]);
-  const double el2 = el * el, er2 = er * er, eb2 = eb * eb, et2 = et * et;
-  beta[1] = el2 + eb2;
-  beta[2] = er2 + eb2;
-  beta[3] = el2 + et2;
-  beta[4] = er2 + et2;
-  const double a = (to_f64(fabs(u[1])) + to_f64(fabs(u[3])) + to_f64(fabs(u[4])) +
-                    to_f64(fabs(u[5])) + to_f64(fabs(u[7]))) * 0.2;
-  uave = a * a;
-}
-
 // The combined polynomial (Eq. 2.23) a0 p_0 + sum_m b_m p_m in monomial coefficients C;
 // om = 1 - a0 (formed in double by the caller: the constant term of the p_m is u5).
 template <typename R>
@@ -451,41 +391,6 @@ __device__ __forceinline__ void combine2d(const R (&c)[15], const R (&u)[9], R a
   C[2] = a0 * c[2] + (b1 + b2) * db + (b3 + b4) * dtp;
 #pragma unroll
   for (int n = 3; n < 15; ++n) C[n] = a0 * c[n];
-}
-
-// One field, Steps 2-3 and the combination, from the Appendix coefficients c of p_0 and the
-// averages u[1], u[3], u[4], u[5], u[7] of cells 2, 4, 5, 6, 8 (the other entries of u are
-// not read): combined monomial coefficients C[15].
-// WMODE 0: the weights by nonlinear_weights (product form, direct formula where it does not
-// apply; `ok` cleared where the direct formula was used); 1: the product form alone, without
-// a branch, `ok` cleared where it does not apply (the caller redoes those cells with WMODE 2);
-// 2: the direct formula.
-template <typename R, int WMODE = 0>
-__device__ __forceinline__ void recon2d_from_coeffs(const R (&c)[15], const R (&u)[9],
-                                                    const KProblem& P, R (&C)[15], bool& ok) {
-  double beta[5], uave;
-  beta2d<R>(c, u, beta, uave);
-  double a0d, bm[5];
-  if constexpr (WMODE == 0) ok &= nonlinear_weights<5>(beta, uave, P, a0d, bm);
-  else if constexpr (WMODE == 1) ok &= nonlinear_weights_fast<5>(beta, uave, P, a0d, bm);
-  else nonlinear_weights_direct<5>(beta, uave, P, a0d, bm);
-  combine2d<R>(c, u, from_f64<R>(a0d), from_f64<R>(1.0 - a0d), from_f64<R>(bm[1]),
-               from_f64<R>(bm[2]), from_f64<R>(bm[3]), from_f64<R>(bm[4]), C);
-}
-// Steps 1-3 of one field from its stencil (u[9] averages, v[4] / w[4] first moments of cells
-// 2, 4, 6, 8).
-template <typename R, int WMODE = 0>
-__device__ __forceinline__ void recon2d_coeffs(const R (&u)[9], const R (&v)[4], const R (&w)[4],
-                                               const KProblem& P, R (&C)[15], bool& ok) {
-  R c[15];
-  coeffs2d<R>(u, v, w, c);
-  recon2d_from_coeffs<R, WMODE>(c, u, P, C, ok);
-}
-template <typename R>
-__device__ __forceinline__ void recon2d_coeffs(const R (&u)[9], const R (&v)[4], const R (&w)[4],
-                                               const KProblem& P, R (&C)[15]) {
-  bool ok = true;
-  recon2d_coeffs<R, 0>(u, v, w, P, C, ok);
 }
 
 // Gauss node sqrt(15)/10 and powers

@@ -19,6 +19,7 @@ namespace c64 {
 constexpr double S1 = 0.38729833462074168852;  // sqrt(15)/10, the outer Gauss node
 constexpr double S2 = 0.15, S3 = S1 * 0.15, S4 = 0.0225;
 
+// S1 .. S4 are those of the coordinates: scaled here, 1 in namespace plain
 #define HW_C64_CONSTANTS(X)                                                                   \
   X(ONE, 1.0) X(MZERO, -0.0)                                                                  \
   /* beta_0 */                                                                                \
@@ -58,19 +59,31 @@ static __constant__ double c64_constants[kStatic] = {
     HW_C64_CONSTANTS(X)
 #undef X
 };
+// the same in unscaled coordinates, for the FP32-bulk kernels, whose smoothness indicators and
+// weights are evaluated in FP64 by the functions below
+namespace plain {
+constexpr double S1 = 1.0, S2 = 1.0, S3 = 1.0, S4 = 1.0;
+static __constant__ double constants[kStatic] = {
+#define X(name, value) (value),
+    HW_C64_CONSTANTS(X)
+#undef X
+};
+}  // namespace plain
 constexpr int kTable = (kCount + 7) / 8 * 8;  // doubles of shared memory
 
 #define K(name) o.k<c64::k##name>()
 
 // the table of an item (visible after the caller's next __syncthreads)
+template <bool SCALED = true>
 __device__ __forceinline__ void fill_table(double* tab, const KProblem& P) {
   const int t = threadIdx.x;
-  for (int n = t; n < kStatic; n += blockDim.x) tab[n] = c64_constants[n];
+  for (int n = t; n < kStatic; n += blockDim.x)
+    tab[n] = SCALED ? c64_constants[n] : plain::constants[n];
   if (t == 0) {
     tab[kEPS] = 25.0 * P.eps;  // d_m is scaled by 25, the squared divisor of u_ave
     tab[kGLO] = P.glo;
     tab[kG0] = P.g0[1];
-    tab[kSGLO] = S1 * P.glo;
+    tab[kSGLO] = (SCALED ? S1 : 1.0) * P.glo;
     tab[kGM1] = P.gm1;
     tab[kHGM1] = -0.5 * P.gm1;
     tab[kGAM] = P.gam;
@@ -120,59 +133,113 @@ struct Factors {
   double a0, l, r, b, t;
 };
 
-// Eq. 2.20-2.22 from beta_0 and the one-sided differences e = {el, er, eb, et}; w5 the field's
-// cell average (zero where ZERO_MEAN).  The product form of hweno_device.cuh's
-// nonlinear_weights_fast, in the sums the combination needs and with d_m scaled by 25 (the
-// squared divisor of u_ave); the direct formula where the products leave the double range.
+// the sum of |averages| of cells 2, 4, 5, 6, 8 (5 sqrt(u_ave)) from the cell's own, w5, and the
+// one-sided differences; w5 = 0 where ZERO_MEAN
 template <bool ZERO_MEAN>
-__device__ __forceinline__ bool factors(const Ops& o, double bt0, const double (&e)[4], double w5,
-                                        const KProblem& P, Factors& F) {
-  const double el2 = o.mul(e[0], e[0]), er2 = o.mul(e[1], e[1]), eb2 = o.mul(e[2], e[2]),
-               et2 = o.mul(e[3], e[3]);
-  const double b1 = o.add(el2, eb2), b2 = o.add(er2, eb2), b3 = o.add(el2, et2),
-               b4 = o.add(er2, et2);
-  const double s = o.add(o.add(fabs(o.sub(bt0, b1)), fabs(o.sub(bt0, b2))),
-                         o.add(fabs(o.sub(bt0, b3)), fabs(o.sub(bt0, b4))));
-  const double tau = o.mul(o.mul(K(W_TAU), s), s);  // 25 tau
-  double a;
+__device__ __forceinline__ double average_sum(const Ops& o, const double (&e)[4], double w5) {
   if constexpr (ZERO_MEAN)
-    a = o.add(o.add(fabs(e[0]), fabs(e[1])), o.add(fabs(e[2]), fabs(e[3])));
+    return o.add(o.add(fabs(e[0]), fabs(e[1])), o.add(fabs(e[2]), fabs(e[3])));
   else
-    a = o.add(o.add(o.add(fabs(o.sub(w5, e[0])), fabs(o.add(w5, e[1]))),
-                    o.add(fabs(o.sub(w5, e[2])), fabs(o.add(w5, e[3])))), fabs(w5));
-  double ua = o.mul(a, a);  // 25 u_ave
-  if (P.wmode == 1) ua = 25.0;
-  const double eps = K(EPS);
-  const double d0 = fma(bt0, ua, eps), d1 = fma(b1, ua, eps), d2 = fma(b2, ua, eps),
-               d3 = fma(b3, ua, eps), d4 = fma(b4, ua, eps);
-  const double p12 = o.mul(d1, d2), p34 = o.mul(d3, d4);
-  const double D0 = o.mul(p12, p34), D = o.mul(D0, d0);
-  const double A = o.mul(d0, p34), B = o.mul(d0, p12);  // D1 = A d2, D2 = A d1, D3 = B d4, D4 = B d3
-  const double q12 = o.mul(A, o.add(d1, d2)), q34 = o.mul(B, o.add(d3, d4));
-  const double q13 = fma(A, d2, o.mul(B, d4)), q24 = fma(A, d1, o.mul(B, d3));
-  const double q = o.add(q12, q34);
-  const double N0 = fma(tau, D0, D);
-  const double S = fma(tau, fma(K(GLO), q, o.mul(K(G0), D0)), D);
-  const long long eD = (__double_as_longlong(D) >> 52) & 0x7ff;
-  const long long eS = (__double_as_longlong(S) >> 52) & 0x7ff;
-  const bool ok = eD > 64 && eD < 2047 - 64 && eS > 64 && eS < 2047 - 64;
+    return o.add(o.add(o.add(fabs(o.sub(w5, e[0])), fabs(o.add(w5, e[1]))),
+                       o.add(fabs(o.sub(w5, e[2])), fabs(o.add(w5, e[3])))), fabs(w5));
+}
+
+// Eq. 2.20-2.22 from beta_0, the one-sided differences e = {el, er, eb, et} and a, the average
+// sum: the product form of hweno_device.cuh's nonlinear_weights_fast with d_m scaled by 25 (the
+// squared divisor of u_ave), as far as its users share it.
+struct Products {
+  double b1, b2, b3, b4;  // beta_m of the linear polynomials
+  double D0, A, B, d1, d2, d3, d4;  // D_1 = A d2, D_2 = A d1, D_3 = B d4, D_4 = B d3
+  double N0, inv, tau;                       // a0 = N0 inv
+  bool ok;  // the products stay in the double range
+
+  // q = D_1 + .. + D_4 by sum(*this)
+  template <class Sum>
+  __device__ __forceinline__ void set(const Ops& o, double bt0, const double (&e)[4], double a,
+                                      const KProblem& P, Sum sum) {
+    const double el2 = o.mul(e[0], e[0]), er2 = o.mul(e[1], e[1]), eb2 = o.mul(e[2], e[2]),
+                 et2 = o.mul(e[3], e[3]);
+    b1 = o.add(el2, eb2);
+    b2 = o.add(er2, eb2);
+    b3 = o.add(el2, et2);
+    b4 = o.add(er2, et2);
+    const double s = o.add(o.add(fabs(o.sub(bt0, b1)), fabs(o.sub(bt0, b2))),
+                           o.add(fabs(o.sub(bt0, b3)), fabs(o.sub(bt0, b4))));
+    tau = o.mul(o.mul(K(W_TAU), s), s);  // 25 tau
+    double ua = o.mul(a, a);             // 25 u_ave
+    if (P.wmode == 1) ua = 25.0;
+    const double eps = K(EPS);
+    const double d0 = fma(bt0, ua, eps);
+    d1 = fma(b1, ua, eps);
+    d2 = fma(b2, ua, eps);
+    d3 = fma(b3, ua, eps);
+    d4 = fma(b4, ua, eps);
+    const double p12 = o.mul(d1, d2), p34 = o.mul(d3, d4);
+    D0 = o.mul(p12, p34);
+    const double D = o.mul(D0, d0);
+    A = o.mul(d0, p34);
+    B = o.mul(d0, p12);
+    const double q = sum(*this);
+    N0 = fma(tau, D0, D);
+    const double S = fma(tau, fma(K(GLO), q, o.mul(K(G0), D0)), D);
+    const int eD = (__double2hiint(D) >> 20) & 0x7ff, eS = (__double2hiint(S) >> 20) & 0x7ff;
+    ok = eD > 64 && eD < 2047 - 64 && eS > 64 && eS < 2047 - 64;
+    inv = rcp_in_range(o, S);
+  }
+};
+
+// The factors; false where the products left the double range and the direct formula was used.
+__device__ __forceinline__ bool factors(const Ops& o, double bt0, const double (&e)[4], double a,
+                                        const KProblem& P, Factors& F) {
+  Products p;
+  double q12, q34, q13, q24;
+  p.set(o, bt0, e, a, P, [&](const Products& x) {
+    q12 = o.mul(x.A, o.add(x.d1, x.d2));
+    q34 = o.mul(x.B, o.add(x.d3, x.d4));
+    q13 = fma(x.A, x.d2, o.mul(x.B, x.d4));
+    q24 = fma(x.A, x.d1, o.mul(x.B, x.d3));
+    return o.add(q12, q34);
+  });
   const bool lin = P.wmode == 2;
-  const double inv = rcp_in_range(o, S);
-  const double k = o.mul(K(SGLO), o.mul(tau, inv));
-  const double k0 = o.mul(K(MTWO), o.mul(k, D0));
-  F.a0 = lin ? 1.0 : o.mul(N0, inv);
+  const double k = o.mul(K(SGLO), o.mul(p.tau, p.inv));
+  const double k0 = o.mul(K(MTWO), o.mul(k, p.D0));
+  F.a0 = lin ? 1.0 : o.mul(p.N0, p.inv);
   F.l = lin ? 0.0 : fma(k, q13, k0);
   F.r = lin ? 0.0 : fma(k, q24, k0);
   F.b = lin ? 0.0 : fma(k, q12, k0);
   F.t = lin ? 0.0 : fma(k, q34, k0);
-  if (ok || lin) return true;
-  const double beta[5] = {bt0, b1, b2, b3, b4};
+  if (p.ok || lin) return true;
+  const double beta[5] = {bt0, p.b1, p.b2, p.b3, p.b4};
   double bm[5];
   nonlinear_weights_direct<5>(beta, 0.04 * (a * a), P, F.a0, bm);
   F.l = S1 * (bm[1] + bm[3]);
   F.r = S1 * (bm[2] + bm[4]);
   F.b = S1 * (bm[1] + bm[2]);
   F.t = S1 * (bm[3] + bm[4]);
+  return false;
+}
+// The same as a0 and the single b_1..b_4, in unscaled coordinates.
+__device__ __forceinline__ bool weights(const Ops& o, double bt0, const double (&e)[4], double a,
+                                        const KProblem& P, double& a0, double (&b)[5]) {
+  Products p;
+  double D1, D2, D3, D4;
+  p.set(o, bt0, e, a, P, [&](const Products& x) {
+    D1 = o.mul(x.A, x.d2);
+    D2 = o.mul(x.A, x.d1);
+    D3 = o.mul(x.B, x.d4);
+    D4 = o.mul(x.B, x.d3);
+    return o.add(o.add(D1, D2), o.add(D3, D4));
+  });
+  const bool lin = P.wmode == 2;
+  const double k = o.mul(K(GLO), o.mul(p.tau, p.inv)), k0 = -o.mul(k, p.D0);
+  a0 = lin ? 1.0 : o.mul(p.N0, p.inv);
+  b[1] = lin ? 0.0 : fma(k, D1, k0);
+  b[2] = lin ? 0.0 : fma(k, D2, k0);
+  b[3] = lin ? 0.0 : fma(k, D3, k0);
+  b[4] = lin ? 0.0 : fma(k, D4, k0);
+  if (p.ok || lin) return true;
+  const double beta[5] = {bt0, p.b1, p.b2, p.b3, p.b4};
+  nonlinear_weights_direct<5>(beta, 0.04 * (a * a), P, a0, b);
   return false;
 }
 

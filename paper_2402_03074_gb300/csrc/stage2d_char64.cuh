@@ -109,7 +109,7 @@ struct Char64Cell {
       coefficients(o, [this](int n) { return w1p[n * T]; }, dW, C);
       Factors F;
       const double mean = o.sub(w0[0 * WC + 1], X5);
-      fast &= factors<false>(o, beta0(o, C), dW, mean, P, F);
+      fast &= factors(o, beta0(o, C), dW, average_sum<false>(o, dW, mean), P, F);
 #pragma unroll
       for (int n = 1; n < 15; ++n) C[n] = o.mul(C[n], F.a0);
       C[1] = fma(F.r, dW[1], fma(F.l, dW[0], C[1]));
@@ -165,7 +165,7 @@ struct Char64Cell {
         for (int n = 1; n < 15; ++n) C[n] = fma(-hic, cN[(n - 1) * T], cX[(n - 1) * T]);
 #pragma unroll
         for (int n = 0; n < 4; ++n) e[n] = fma(-hic, eN[n], dX[n]);
-        fast &= factors<false>(o, beta0(o, C), e, w5, P, F0);
+        fast &= factors(o, beta0(o, C), e, average_sum<false>(o, e, w5), P, F0);
         s0x = fma(F0.r, e[1], o.mul(F0.l, e[0]));
         s0y = fma(F0.t, e[3], o.mul(F0.b, e[2]));
       }
@@ -175,7 +175,7 @@ struct Char64Cell {
         for (int n = 1; n < 15; ++n) C[n] = fma(hic, cN[(n - 1) * T], cX[(n - 1) * T]);
 #pragma unroll
         for (int n = 0; n < 4; ++n) e[n] = fma(hic, eN[n], dX[n]);
-        fast &= factors<false>(o, beta0(o, C), e, w5, P, F3);
+        fast &= factors(o, beta0(o, C), e, average_sum<false>(o, e, w5), P, F3);
         s3x = fma(F3.r, e[1], o.mul(F3.l, e[0]));
         s3y = fma(F3.t, e[3], o.mul(F3.b, e[2]));
       }
@@ -199,7 +199,7 @@ struct Char64Cell {
 #pragma unroll
       for (int n = 1; n < 15; ++n) PT[n] = cT[(n - 1) * T];
       Factors F;
-      fast &= factors<true>(o, beta0(o, PT), eT, 0.0, P, F);
+      fast &= factors(o, beta0(o, PT), eT, average_sum<true>(o, eT, 0.0), P, F);
 #pragma unroll
       for (int n = 1; n < 15; ++n) PT[n] = o.mul(PT[n], F.a0);
       PT[1] = fma(F.r, eT[1], fma(F.l, eT[0], PT[1]));

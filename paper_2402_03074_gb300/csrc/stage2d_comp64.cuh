@@ -40,7 +40,7 @@ struct Comp64Cell {
       coefficients(o, [&s](int n) { return s[n]; }, e, C);
       const double mean = w0[3 * a * WC + 1];
       Factors F;
-      fast &= factors<false>(o, beta0(o, C), e, mean, P, F);
+      fast &= factors(o, beta0(o, C), e, average_sum<false>(o, e, mean), P, F);
 #pragma unroll
       for (int n = 1; n < 15; ++n) C[n] = o.mul(C[n], F.a0);
       C[1] = fma(F.r, e[1], fma(F.l, e[0], C[1]));

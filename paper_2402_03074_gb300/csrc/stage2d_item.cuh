@@ -76,8 +76,40 @@ constexpr size_t smem_bytes2d() {
   if constexpr (sizeof(R) == sizeof(double))
     return smem_bytes_tile64<EQ, CHAR, BW, kTileRows<R, BW>>();
   constexpr int BY = kTileRows<R, BW>;
-  return sizeof(R) * ((BY + 2) * 3 * NC * (BW + 2) + (6 + 2) * NC * BW * BY +
+  return sizeof(double) * c64::kTable +
+         sizeof(R) * ((BY + 2) * 3 * NC * (BW + 2) + (6 + 2) * NC * BW * BY +
                       6 * NC * BW * (BY + 1));
+}
+
+// Steps 2 and 3 of one field in FP64 from its FP32 Appendix coefficients c and averages u (of
+// cells 2, 4, 5, 6, 8 are read), by the operations of recon64.cuh in unscaled coordinates: beta_0
+// as in the FP64 kernels, the weights in the product form.  On return c is the combined
+// polynomial (Eq. 2.23) a0 p_0 + sum_m b_m p_m, formed in FP32 from the rounded a0, 1 - a0
+// and b_m.  Returns false where the direct formula was needed.
+//
+// These operations bound the FP32-bulk kernels (the SM takes an FP64 instruction of a warp in 16
+// clocks, FP32 ones in a quarter).  93 per field as three-register FMAs (f64_ops.cuh) instead of
+// 117 in plain operators: 2048^2 step 24.6 -> 22.1 ms.  One evaluation of the entropy field for
+// both passes would take 20.3 ms, but the passes' FP32 coefficients of it round differently, and
+// the results would move by that.
+template <typename R>
+__device__ __forceinline__ bool weigh_field(const Ops& o, const R (&u)[9], const KProblem& P,
+                                            R (&c)[15]) {
+  double d[15];
+#pragma unroll
+  for (int n = 1; n < 15; ++n) d[n] = to_f64(c[n]);
+  const double e[4] = {to_f64(u[4] - u[3]), to_f64(u[5] - u[4]), to_f64(u[4] - u[1]),
+                       to_f64(u[7] - u[4])};
+  const double a = o.add(o.add(o.add(to_f64(fabs(u[1])), to_f64(fabs(u[3]))),
+                               o.add(to_f64(fabs(u[4])), to_f64(fabs(u[5])))),
+                         to_f64(fabs(u[7])));
+  double a0, bm[5];
+  const bool fast = c64::weights(o, c64::beta0(o, d), e, a, P, a0, bm);
+  const R f0 = from_f64<R>(a0), om = from_f64<R>(o.sub(o.one, a0));
+  const R b1 = from_f64<R>(bm[1]), b2 = from_f64<R>(bm[2]), b3 = from_f64<R>(bm[3]),
+          b4 = from_f64<R>(bm[4]);
+  combine2d<R>(c, u, f0, om, b1, b2, b3, b4, c);
+  return fast;
 }
 
 template <int EQ, bool CHAR, typename R, int BX, int BY>
@@ -92,7 +124,8 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
   const int tx = t % BX, ty = t / BX;  // ty is uniform over a warp
   // rows of the stage input for the reconstruction of the tile's rows, row r in slot
   // (r - j0 + 2) mod NR
-  R* win = reinterpret_cast<R*>(smem);                  // [NR][NA][WC]
+  c64::fill_table<false>(smem, P);
+  R* win = reinterpret_cast<R*>(smem + c64::kTable);    // [NR][NA][WC]
   // x-face exchange of the thread's row, [NC][3][2][BX]: the left trace u and its flux f of every
   // thread's cell; the face flux at the left face of thread x's cell then overwrites the u
   // slot x (its only reader, thread x - 1, has read it by then)
@@ -142,6 +175,7 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
 #pragma unroll 1
   for (int r = j0 - 2 + ty; r <= j0 - 1 + BY && r <= j1 + 1; r += BY) load_row(r);
   __syncthreads();
+  const Ops o = make_ops<c64::kONE, c64::kMZERO>(smem, S.k);
   // the threads of a row wait for each other (named barrier of the row; a warp on its own)
   auto row_sync = [&]() {
     if constexpr (BX == 32) __syncwarp();
@@ -293,35 +327,13 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
                 w[e] = Ww[e][f];
               }
             };
-            // per field: coefficients, FP64 smoothness indicators and weights (the branch-free
-            // product form), combination and evaluation.  The fields are taken in pairs whose
-            // two FP64 weight chains share a basic block (the direct formula, for the rare
-            // cells that need it, after both), which hides part of their latency: 9.10 ms
-            // against 9.20-9.27 ms per 2048^2 stage
 #pragma unroll
-            for (int f0 = 0; f0 < 4; f0 += 2) {
-              bool ok = true;
-              R C0[15], C1[15];
-              {
-                R u[9], v[4], w[4];
-                field(f0, u, v, w);
-                recon2d_coeffs<R, 1>(u, v, w, P, C0, ok);
-              }
-              {
-                R u[9], v[4], w[4];
-                field(f0 + 1, u, v, w);
-                recon2d_coeffs<R, 1>(u, v, w, P, C1, ok);
-              }
-              if (!ok) {
-                fast_weights = false;
-                R u[9], v[4], w[4];
-                field(f0, u, v, w);
-                recon2d_coeffs<R, 2>(u, v, w, P, C0, ok);
-                field(f0 + 1, u, v, w);
-                recon2d_coeffs<R, 2>(u, v, w, P, C1, ok);
-              }
-              evaluate(f0, C0);
-              evaluate(f0 + 1, C1);
+            for (int f = 0; f < 4; ++f) {
+              R u[9], v[4], w[4], C[15];
+              field(f, u, v, w);
+              coeffs2d<R>(u, v, w, C);
+              fast_weights &= weigh_field<R>(o, u, P, C);
+              evaluate(f, C);
             }
           }
           R cons[16][4];
@@ -373,7 +385,8 @@ __device__ __forceinline__ void stage2d_mixed_item(const KProblem& P, const KSta
             w[e] = Wv(c * NM + 2, 2 * e + 1);
           }
           R C[15];
-          recon2d_coeffs<R, 0>(u, v, w, P, C, fast_weights);
+          coeffs2d<R>(u, v, w, C);
+          fast_weights &= weigh_field<R>(o, u, P, C);
           R ea[3], eb[3], in[9];
           eval_xpass(C, ea, eb, in);
 #pragma unroll
