@@ -16,7 +16,7 @@ LIB = os.path.join(HERE, "libhweno.so")
 SOURCES = ["stage2d.cu", "stage2d_w96.cu", "stage2d_w64.cu", "stage2d_w192.cu", "stage2d_w32.cu",
            "stage1d.cu",
            "batch.cu", "static_batch.cu", "engine.cu", "server.cu", "tune.cu", "peaks.cu"]
-HEADERS = ["hweno_device.cuh", "f64_ops.cuh", "launch.h", "server.h", "batch.h", "geometry.h",
+HEADERS = ["hweno_device.cuh", "f64_ops.cuh", "rcp64.h", "launch.h", "server.h", "batch.h", "geometry.h",
            "stage1d_item.cuh", "stage1d_lanes64.cuh",
            "stage2d_item.cuh", "recon64.cuh", "stage2d_char64.cuh",
            "stage2d_comp64.cuh", "stage2d_tile64.cuh", "stage2d_impl.cuh"]

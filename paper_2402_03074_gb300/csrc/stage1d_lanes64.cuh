@@ -92,15 +92,6 @@ __device__ __forceinline__ void fill_table(double* tab, const KProblem& P) {
 }
 #define K(name) o.k<l64::k##name>()
 
-// 1/sqrt(x) of a positive normal double: the hardware's 20-bit value y refined by one third-order
-// step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2 (the new residual is below 2^-59).
-__device__ __forceinline__ double rsqrt_refined(const Ops& o, double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-o.mul(x, y), y, o.one);
-  return fma(o.mul(y, e), fma(K(RS2), e, K(HALF)), y);
-}
-
 // The factors of the combined polynomial (Eq. 2.12): a0 of p_0 and b1, b2 of the slopes dl, dr
 // (the product form of nonlinear_weights_fast, d_m scaled by 9; the direct formula where it
 // does not apply).
@@ -148,7 +139,7 @@ struct Frame1 {
     q2h = o.mul(o.mul(K(HALF), vel), vel);
     const double p = o.mul(K(GM1), fma(-U0, q2h, U2));
     const double c2 = o.mul(o.mul(K(GAM), p), ir);
-    const double rc = rsqrt_refined(o, c2);
+    const double rc = rsqrt_refined(o, c2, K(HALF), K(RS2));
     cs = o.mul(c2, rc);
     H = o.mul(o.add(U2, p), ir);
     b1h = -o.mul(o.mul(K(HGM1), rc), rc);
@@ -246,7 +237,7 @@ __device__ __forceinline__ double speed64(const Ops& o, const double (&ua)[3], b
   const double e = fma(-o.mul(K(HALF), ua[1]), vn, ua[2]);  // internal energy density
   const double c2 = o.mul(o.mul(o.mul(K(GAM), K(GM1)), e), ir);
   ok &= ua[0] > 0.0 && e > 0.0 && finite_bits(e);
-  return fma(c2, rsqrt_refined(o, c2), fabs(vn));
+  return fma(c2, rsqrt_refined(o, c2, K(HALF), K(RS2)), fabs(vn));
 }
 
 }  // namespace l64

@@ -49,7 +49,7 @@ struct Char64Cell {
     {
       const double U0 = w0[0 * WC + 1], U1 = w0[3 * WC + 1], U2 = w0[6 * WC + 1],
                    U3 = w0[9 * WC + 1];
-      const double ir = rcp_any(o, U0);
+      const double ir = rcp_any(U0);
       vx = o.mul(U1, ir);
       vy = o.mul(U2, ir);
       q2h = o.mul(K(HALF), fma(vx, vx, o.mul(vy, vy)));
@@ -227,7 +227,7 @@ struct Char64Cell {
           const double r = o.add(w1p[(6 * DIR + 3 * side + g) * T], X[side][g]);
           double mn, mt, E;
           conserved(r, Q[side][g], Y[side][g], X[side][g], mn, mt, E);
-          const double ir = rcp_any(o, r);
+          const double ir = rcp_any(r);
           const double vn = o.mul(mn, ir);
           const double kin = o.mul(fma(mn, mn, o.mul(mt, mt)), ir);
           const double p = fma(hg, kin, o.mul(gm1, E));
@@ -251,7 +251,7 @@ struct Char64Cell {
 #pragma unroll
       for (int g = 0; g < 9; ++g) {
         const double r = o.add(w1p[(12 + g) * T], X[g]);
-        const double ir = rcp_any(o, r);
+        const double ir = rcp_any(r);
         const double wir = o.mul(g == 4 ? wm_ : ((g & 1) ? we : wc), ir);
         const double qa = o.mul(Q[g], wir);
         const double z = fma(Q[g], Q[g], o.mul(Y[g], Y[g]));

@@ -62,7 +62,7 @@ struct Comp64Cell {
       f[0] = o.mul(o.mul(K(HALF), u[0]), u[0]);
     } else {
       constexpr int n = 1 + DIR, t = 2 - DIR;
-      const double ir = rcp_any(o, u[0]);
+      const double ir = rcp_any(u[0]);
       const double vn = o.mul(u[n], ir);
       const double kin = o.mul(fma(u[n], u[n], o.mul(u[t], u[t])), ir);
       const double p = fma(K(HGM1), kin, o.mul(K(GM1), u[3]));
@@ -133,7 +133,7 @@ struct Comp64Cell {
       const double wc = K(WC), we = K(WE), wm_ = K(WM), gm1 = K(GM1), hg = K(HGM1);
 #pragma unroll
       for (int g = 0; g < 9; ++g) {
-        const double ir = rcp_any(o, u[0][g]);
+        const double ir = rcp_any(u[0][g]);
         const double wir = o.mul(g == 4 ? wm_ : ((g & 1) ? we : wc), ir);
         const double wx = o.mul(u[1][g], wir), wy = o.mul(u[2][g], wir);
         const double kin = o.mul(fma(u[1][g], u[1][g], o.mul(u[2][g], u[2][g])), ir);
