@@ -66,9 +66,12 @@ __device__ __forceinline__ double rcp_any(const Ops& o, double x) {
   return rcp_applies(x) ? rcp_in_range(o, x) : 1.0 / x;
 }
 
-// 1/sqrt(x) of a positive normal double: the hardware's 20-bit value y refined by one third-order
-// step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2 (the new residual is below 2^-59).  half and c38: 1/2, 3/8.
-__device__ __forceinline__ double rsqrt_refined(const Ops& o, double x, double half, double c38) {
+// 1/sqrt(x): the hardware's 20-bit value y refined by one third-order step y (1 + e/2 + 3 e^2/8),
+// e = 1 - x y^2 (the new residual is below 2^-59); the library's where x is near the ends of the
+// range or not positive.  half and c38: 1/2 and 3/8.
+__device__ __forceinline__ double rsqrt_any(const Ops& o, double x, double half, double c38) {
+  const int eb = __double2hiint(x) >> 20;
+  if (eb < 64 || eb > 1983) return rsqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-o.mul(x, y), y, o.one);

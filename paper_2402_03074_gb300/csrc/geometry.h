@@ -94,9 +94,12 @@ inline Geom2D geom2d(int nx, int ny, int bw, int slots, int rows_fixed, int band
   return g;
 }
 
-// ---- Tiles: FP64 bx columns x tile_rows64(bx) rows of threads per block (stage2d_tile64.cuh),
-// six or seven warps, so that one block fills an SM's FP64 unit.
-constexpr int tile_rows64(int bx) { return bx == 32 ? 7 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
+// ---- Tiles: FP64 bx columns x tile_rows64(bx) rows of threads per block (stage2d_tile64.cuh):
+// eight warps, two per scheduler, of 255 registers a thread (96 columns: six, the shared memory's
+// limit).  Against seven and six warps (32 x 7, 64 x 3): 240^2 Euler, 12 steps, 11.55 -> 10.05 ms,
+// 240^2 Burgers, 48 steps, 7.98 -> 7.00 ms, eight-solve batch 7.41 -> 6.78 ms, 768^2 component-wise
+// 5.30 -> 5.19 ms; 320^2 (whose chunks of 27 rows fill 7-row steps better) 1.62 -> 1.66 ms.
+constexpr int tile_rows64(int bx) { return bx == 32 ? 8 : bx == 64 ? 4 : bx == 96 ? 2 : 1; }
 // The same for the FP32-bulk kernels: six warps per block, two blocks per SM (128 columns: four
 // warps, three blocks).
 constexpr int tile_rows32(int bx) { return bx == 32 ? 6 : bx == 64 ? 3 : bx == 96 ? 2 : 1; }
@@ -120,9 +123,10 @@ inline double tile_time64(int warps, int by, int rows, int blocks, double step) 
 
 // The default tile of a grid: over the widths bx[0..n-1] (with slots[] resident blocks per GPU
 // each, on `sms` SMs) and the chunk heights (or one segment per resident block), the launch of
-// least time.  240^2 FP64: 32 x 7, 8 bands x 19 chunks of 13 rows (1.00 ms per three stages,
-// 1.06 in 64 x 3 tiles, 1.45 in rows of 192); 2048^2 FP64: 96 x 2, 22 bands in 152 segments of 297
-// band-rows (56.5 ms; 57.3 in 32 x 7, whose ring columns cost 7 % instead of 2 %).
+// least time.  240^2 FP64: 32 x 8, 8 bands x 19 chunks of 13 rows (0.84 ms per three stages); 2048^2
+// FP64: 96 x 2, 22 bands in 152 segments of 297 band-rows (54.5 ms; 54.2 in 64 x 4 and 54.5 in 32 x 8,
+// whose eight warps make up for ring columns of 3 and 7 % instead of 2 %); 320^2: 32 x 8 in
+// chunks of 25 rows, the last step with three rows (1.66 ms; 1.68 in 64 x 4).
 struct Tile64 {
   int bx;
   int rows;  // output rows per chunk; < -1: segments of -rows band-rows

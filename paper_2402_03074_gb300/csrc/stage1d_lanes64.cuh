@@ -139,7 +139,7 @@ struct Frame1 {
     q2h = o.mul(o.mul(K(HALF), vel), vel);
     const double p = o.mul(K(GM1), fma(-U0, q2h, U2));
     const double c2 = o.mul(o.mul(K(GAM), p), ir);
-    const double rc = rsqrt_refined(o, c2, K(HALF), K(RS2));
+    const double rc = rsqrt_any(o, c2, K(HALF), K(RS2));
     cs = o.mul(c2, rc);
     H = o.mul(o.add(U2, p), ir);
     b1h = -o.mul(o.mul(K(HGM1), rc), rc);
@@ -237,7 +237,7 @@ __device__ __forceinline__ double speed64(const Ops& o, const double (&ua)[3], b
   const double e = fma(-o.mul(K(HALF), ua[1]), vn, ua[2]);  // internal energy density
   const double c2 = o.mul(o.mul(o.mul(K(GAM), K(GM1)), e), ir);
   ok &= ua[0] > 0.0 && e > 0.0 && finite_bits(e);
-  return fma(c2, rsqrt_refined(o, c2, K(HALF), K(RS2)), fabs(vn));
+  return c2 > 0.0 ? fma(c2, rsqrt_any(o, c2, K(HALF), K(RS2)), fabs(vn)) : fabs(vn);
 }
 
 }  // namespace l64

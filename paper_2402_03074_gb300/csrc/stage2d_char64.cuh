@@ -55,7 +55,7 @@ struct Char64Cell {
       q2h = o.mul(K(HALF), fma(vx, vx, o.mul(vy, vy)));
       p5 = o.mul(K(GM1), fma(-U0, q2h, U3));
       c2 = o.mul(o.mul(K(GAM), p5), ir);
-      const double rc = rsqrt(c2);
+      const double rc = rsqrt_any(o, c2, K(HALF), K(RS2));
       c = o.mul(c2, rc);
       h = fma(o.add(U3, p5), ir, -q2h);
       hic = o.mul(K(HALF), rc);

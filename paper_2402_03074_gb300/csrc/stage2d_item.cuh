@@ -25,7 +25,7 @@ template <typename R, int BW>
 constexpr int kThreads2D = BW * kTileRows<R, BW>;
 
 // Resident blocks per SM the 2D stage kernels are compiled for: the FP64 Euler kernels take the
-// register file and the shared memory with one block (two of 128 threads would not fit), the
+// register file and the shared memory with one block of 256 threads, the
 // scalar FP64 ones two; the FP32-bulk kernels twelve warps (at most 168 registers per thread),
 // which hides more of the FP64 latency of their weight evaluation.
 template <int EQ, typename R, int BW>

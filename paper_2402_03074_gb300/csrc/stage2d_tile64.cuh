@@ -12,16 +12,17 @@
 // one step later.  Redundant work is the two ring columns per band and the y traces of the two
 // ring rows per chunk.
 //
-// Why BY rows at once: an SM needs about six warps to keep its FP64 unit busy (a warp alone gets
+// Why BY rows at once: an SM needs six to eight warps to keep its FP64 unit busy (a warp alone gets
 // one FP64 instruction in 64 clocks, the SM one in 16), and a chunk of r rows costs r + 0.9 rows
 // of work (the ring rows' y passes).  With one row at a time, six warps are two 96-column blocks
 // each with its own ring rows, and a grid of 240^2 cells in chunks of 3 rows spends a quarter of
-// its work on ring rows and idle lanes; one block of 32 x 7 covers 13 rows in 30 columns.
-// Measured against one row at a time (whole calls; characteristic Euler in two 96-thread blocks
-// per SM, the other classes in 128-thread blocks of the field-by-field arithmetic): 240^2 Euler,
-// 12 steps, 17.3 -> 11.9 ms; 40^2 Euler, 24 steps, 13.6 -> 7.8 ms; 517 x 389 Euler, one step, 3.33
-// -> 3.25 ms; 2048^2 Euler, one step, 56.5 -> 56.3 ms; 240^2 Burgers, 48 steps, 17.0 -> 8.0 ms;
-// 768^2 component-wise Euler, one step, 8.39 -> 5.49 ms.
+// its work on ring rows and idle lanes; one block of 32 x 8 covers 13 rows in 30 columns.
+// Measured (whole calls; before: characteristic Euler one row at a time in two 96-thread blocks
+// per SM, the other classes in 128-thread blocks of the field-by-field arithmetic; then the tiles
+// of six or seven warps; then the present ones, with their reciprocals on integers): 240^2 Euler,
+// 12 steps, 17.3, 11.9, 10.05 ms; 40^2 Euler, 24 steps, 13.6, 7.27, 7.32 ms; 517 x 389 Euler, one
+// step, 3.33, 3.27, 3.15 ms; 2048^2 Euler, one step, 56.5, 56.4, 54.5 ms; 240^2 Burgers, 48 steps,
+// 17.0, 8.05, 7.01 ms; 768^2 component-wise Euler, one step, 8.39, 5.50, 5.19 ms.
 #pragma once
 #include "stage2d_char64.cuh"
 #include "stage2d_comp64.cuh"
@@ -40,12 +41,16 @@ struct Cell64<EQ_EULER, true, T, WC> {
 // Shared memory of a block: the row window [BY + 2][NA][BX + 2]; per thread the x-face exchange
 // (3 NC: flux - a u of the low trace, then the Gauss moments of the face's flux), the high y
 // traces (3 NC, and BX columns more: the tile's last row in turns), the y-face moments (2 NC)
-// and the cell's column; and the table of constants.
+// and the cell's column; and the table of constants.  In the Euler tiles of eight warps the y-face
+// moments lie in the exchange (kSharedFaces; one more barrier between steps): it would be 235 KB.
+template <int EQ, int BX, int BY>
+constexpr bool kSharedFaces = EQ == EQ_EULER && BX * BY == 256;
 template <int EQ, bool CHAR, int BX, int BY>
 constexpr size_t smem_bytes_tile64() {
   using Cell = typename Cell64<EQ, CHAR, BX * BY, BX + 2>::type;
   constexpr int NC = Cell::NC;
-  return sizeof(double) * ((BY + 2) * 3 * NC * (BX + 2) + (8 * NC + Cell::kCols) * BX * BY +
+  return sizeof(double) * ((BY + 2) * 3 * NC * (BX + 2) +
+                           ((kSharedFaces<EQ, BX, BY> ? 6 : 8) * NC + Cell::kCols) * BX * BY +
                            3 * NC * BX + c64::kTable);
 }
 
@@ -63,8 +68,8 @@ __device__ __forceinline__ void stage2d_tile64_item(const KProblem& P, const KSt
   double* win = smem;
   double* xch = win + NR * NA * WC + t;        // [3 NC][T], this thread's column
   double* car = win + NR * NA * WC + NA * T;   // [BY + 1][3 NC][BX]
-  double* fm = car + (BY + 1) * NA * BX;       // [2 NC][T]
-  double* col = fm + 2 * NC * T;               // [kCols][T]
+  double* fm = kSharedFaces<EQ, BX, BY> ? win + NR * NA * WC : car + (BY + 1) * NA * BX;  // [2 NC][T]
+  double* col = car + (BY + 1) * NA * BX + (kSharedFaces<EQ, BX, BY> ? 0 : 2 * NC * T);   // [kCols][T]
   double* tab = col + Cell::kCols * T;
   fill_table(tab, P);
   const int nx = P.nx, ny = P.ny;
@@ -267,7 +272,7 @@ __device__ __forceinline__ void stage2d_tile64_item(const KProblem& P, const KSt
       }
       if constexpr (EQ == EQ_EULER) {
         double s0, s1;
-        bad |= !euler_speeds<2>(P, ua, s0, s1);
+        bad |= !speeds(o, ua, s0, s1);
         if (!bad) {
           wmax0 = fmax(wmax0, s0);
           wmax1 = fmax(wmax1, s1);
@@ -278,6 +283,8 @@ __device__ __forceinline__ void stage2d_tile64_item(const KProblem& P, const KSt
       }
       if (bad) atomicOr(S.status, kStatusNonphysical);
     }
+    if constexpr (kSharedFaces<EQ, BX, BY>)
+      if (jb + BY <= j1) __syncthreads();  // the faces' place is written next (uniform)
   }
 
   // block maxima of the output wave speeds -> one atomic per block and direction

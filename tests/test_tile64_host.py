@@ -39,7 +39,7 @@ int main() {
   return 0;
 }
 """
-BY = {32: 7, 64: 3, 96: 2}
+BY = {32: 8, 64: 4, 96: 2}
 
 
 @pytest.fixture(scope="module")
