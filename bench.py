@@ -44,23 +44,23 @@ ORACLE_FLOPS_STEP_MEAN = (10078.0 + 2 * 10114.0) / 3.0
 FP64_PEAK_TFLOPS_FALLBACK = 1.19
 FP32_PEAK_TFLOPS_FALLBACK = 74.2
 # FP64 arithmetic the fused 2D Euler characteristic kernel executes per cell-stage, from the
-# ncu thread-instruction counts of one 2048^2 launch in its default geometry (96-thread
-# blocks, 22 bands of 94 columns in 303 segments of 149 band-rows;
-# profiles/stage2d_euler_2048_instruction_counts.md) per updated cell less the 2.9 % of
-# redundant ring-cell reconstruction: operations (DFMA + DMUL + DADD) 3447 -> 3351.  The FP64
+# ncu thread-instruction counts of one 2048^2 launch in its default geometry (96 x 2 tiles, 22
+# bands of 94 columns in 152 segments of 297 band-rows;
+# profiles/stage2d_euler_2048_instruction_counts.md) per updated cell less the 2.5 % of
+# redundant ring-cell reconstruction: operations (DFMA + DMUL + DADD) 2394 -> 2335.  The FP64
 # pipe executes one such operation per lane per clock, so its operation rate is half the FMA
 # flop rate.
-FP64_OPS_PER_CELL_STAGE = 3351.0
-# DRAM bytes read + written by the same launch (ncu)
-FP64_STAGE_DRAM_BYTES = 523.6e6 + 708.3e6
+FP64_OPS_PER_CELL_STAGE = 2335.0
+# DRAM bytes read + written by a launch of stage 2 or 3 (ncu)
+FP64_STAGE_DRAM_BYTES = 957.1e6 + 400.6e6
 # FP64 pipe utilisation of the same launch (% of peak sustained, active cycles)
-FP64_PIPE_UTIL_NCU = 0.843
-# FP32-bulk kernel (same workload, ncu): FP64 arithmetic operations per cell-stage (923 per
-# reconstructed cell in its default geometry -- 192-thread blocks, 11 bands of 187 columns in
-# 27 row chunks -- less 2.3 % ring redundancy), FP32 flops, and the launch's DRAM bytes
-FP32BULK_FP64_OPS_PER_CELL_STAGE = 902.0
-FP32BULK_FP32_FLOPS_PER_CELL_STAGE = 3971.0
-FP32BULK_STAGE_DRAM_BYTES = 462.6e6 + 1068.4e6
+FP64_PIPE_UTIL_NCU = 0.905
+# FP32-bulk kernel (same workload, ncu): FP64 arithmetic operations per cell-stage (832 per
+# updated cell in its default geometry, 96 x 2 tiles, less 2.5 % ring redundancy), FP32
+# flops, and the launch's DRAM bytes
+FP32BULK_FP64_OPS_PER_CELL_STAGE = 812.0
+FP32BULK_FP32_FLOPS_PER_CELL_STAGE = 3960.0
+FP32BULK_STAGE_DRAM_BYTES = 979.0e6 + 413.2e6
 ALGO_BYTES_PER_CELL_STAGE = 277.3   # 12 values read + 12 written (+8 V-hat, stage mean), FP64
 
 

@@ -232,8 +232,8 @@ int hweno_stage_batch_static(int n, const hweno_problem* problems, int k,
 
 /* ---- launch-geometry autotuner -------------------------------------------------------- */
 /* Time one fused stage launch of the 2D problem p on a scratch copy of moments_host for each
-   candidate tile shape -- the block width (128, 96, 64 or 192 threads, one per column of a band
-   plus its two ring columns) x the number of bands the columns are split into (the default bands,
+   candidate tile shape -- the block width (128, 96, 64 or 192 columns of threads: a band plus its
+   two ring columns, by one to eight rows) x the number of bands the columns are split into (the default bands,
    and 1.25, 1.5 and 2 times as many as the widest bands of that width) x the height of the
    row chunks a block sweeps (the default one-wave geometry and 8, 16, 32, 64, 128, 256 rows)
    -- then time the closest candidates (at most four, within 3 % of the fastest) again over
@@ -245,12 +245,10 @@ int hweno_stage_batch_static(int n, const hweno_problem* problems, int k,
    candidates are the block width (128 or 32 threads) and the threads per cell (one per cell,
    or -- Euler with the characteristic decomposition -- one lane per characteristic field in
    blocks of 128, 64 or 32 threads); *best_rows receives the block width and *best_bands the
-   threads per cell (1 or 4).  Output pointers may be NULL.  The 2D bands and rows change no
-   result bit (every cell and face is computed by the same code in any decomposition), nor
-   does the block width, except for FP64 Euler with the characteristic decomposition, whose
-   96-thread blocks form the Appendix coefficients of the conserved components once per cell
-   and project them per pass (the same formulas, equal within rounding); the 1D
-   lanes-per-field layout computes the same formulas, equal within rounding. */
+   threads per cell (1 or 4).  Output pointers may be NULL.  The 2D bands, rows and block width
+   change no result bit (every cell and face is computed by the same code in any decomposition),
+   nor do the threads per cell of a 1D problem in FP64; the FP32-bulk 1D layouts compute the same
+   formulas, equal within rounding. */
 int hweno_autotune(hweno_engine* eng, const hweno_problem* p, const double* moments_host,
                    int* best_rows, int* best_bands, double* best_ms);
 /* Save the tuning table as text (one entry per line, with the GPU name); load it back

@@ -64,7 +64,7 @@ __device__ __forceinline__ void dt_update(DevScal* s, double inv_dx, double inv_
 struct TileShape {
   int rows = 0;
   int bands = 0;
-  // block width: 2D 64, 96, 128 or 192 threads (0 = the default); 1D 0 = the default rule,
+  // block width: 2D 32, 64, 96, 128 or 192 columns (0 = the default); 1D 0 = the default rule,
   // else 32, 64 or 128 threads.  1D threads per cell (0 or 1: one thread per cell; 4: one lane per
   // characteristic field, 1D Euler with the characteristic decomposition)
   int width = 0;

@@ -3,9 +3,8 @@
 // The 2D stage kernel's blocks sweep row chunks of a band.  The tile shape trades redundant
 // work against balance and latency hiding: taller chunks waste fewer ring rows, narrower
 // bands more ring columns and lanes, the tile count sets how evenly the blocks fill the SMs,
-// and the block width (64, 96, 128 or 192 threads) sets the resident warps per SM and the idle
-// lanes of a band (the 96-thread characteristic FP64 kernel also forms the coefficients once
-// per cell).  The autotuner times one stage launch of a problem for each candidate shape
+// and the block width (64, 96, 128 or 192 columns) sets the rows of a tile (geometry.h), the
+// resident warps per SM and the idle lanes of a band.  The autotuner times one stage launch of a problem for each candidate shape
 // (block width x band count x chunk height) on a scratch copy of the caller's moments (with
 // dt = 0, so the copy does not evolve), times the closest few again over whole three-stage
 // sequences, and keeps the fastest in a process-wide table keyed by (equation,
