@@ -47,20 +47,21 @@ FP32_PEAK_TFLOPS_FALLBACK = 74.2
 # ncu thread-instruction counts of one 2048^2 launch in its default geometry (96 x 2 tiles, 22
 # bands of 94 columns in 152 segments of 297 band-rows;
 # profiles/stage2d_euler_2048_instruction_counts.md) per updated cell less the 2.5 % of
-# redundant ring-cell reconstruction: operations (DFMA + DMUL + DADD) 2394 -> 2335.  The FP64
+# redundant ring-cell reconstruction: operations (DFMA + DMUL + DADD) of stage 1, the timed
+# launch, 2370 -> 2312 (2335 in stages 2 and 3).  The FP64
 # pipe executes one such operation per lane per clock, so its operation rate is half the FMA
 # flop rate.
-FP64_OPS_PER_CELL_STAGE = 2335.0
-# DRAM bytes read + written by a launch of stage 2 or 3 (ncu)
-FP64_STAGE_DRAM_BYTES = 957.1e6 + 400.6e6
+FP64_OPS_PER_CELL_STAGE = 2312.0
+# DRAM bytes read + written by the same launch (ncu)
+FP64_STAGE_DRAM_BYTES = 499.4e6 + 661.5e6
 # FP64 pipe utilisation of the same launch (% of peak sustained, active cycles)
-FP64_PIPE_UTIL_NCU = 0.905
+FP64_PIPE_UTIL_NCU = 0.929
 # FP32-bulk kernel (same workload, ncu): FP64 arithmetic operations per cell-stage (832 per
-# updated cell in its default geometry, 96 x 2 tiles, less 2.5 % ring redundancy), FP32
-# flops, and the launch's DRAM bytes
+# updated cell in its default geometry, 96 x 2 tiles, less 2.5 % ring redundancy; stages 2 and
+# 3), FP32 flops, and the DRAM bytes of a stage 1 launch
 FP32BULK_FP64_OPS_PER_CELL_STAGE = 812.0
 FP32BULK_FP32_FLOPS_PER_CELL_STAGE = 3960.0
-FP32BULK_STAGE_DRAM_BYTES = 979.0e6 + 413.2e6
+FP32BULK_STAGE_DRAM_BYTES = 522.9e6 + 688.4e6
 ALGO_BYTES_PER_CELL_STAGE = 277.3   # 12 values read + 12 written (+8 V-hat, stage mean), FP64
 
 
