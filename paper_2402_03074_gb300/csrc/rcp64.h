@@ -45,11 +45,11 @@ HW_RCP64 double rcp64_refine(double x, double y) {
     Y <<= 1;
     top -= 0x100000u;
   }
-  const long long e = -(long long)(M * Y);                  // 2^73 e: the product's upper bits are known
+  const long long e = -(long long)(M * Y);  // 2^73 e: the product's upper bits are known
   const int eh = (int)(e >> 24);
-  const long long e2 = e + (((long long)eh * eh) >> 25);    // 2^73 (e + e^2)
-  const long long corr = ((long long)Y * (e2 >> 13)) >> 25; // 2^35 Y (e + e^2)
-  const unsigned long long Z = ((unsigned long long)Y << 35) + (unsigned long long)corr;     // 56 bits
+  const long long e2 = e + (((long long)eh * eh) >> 25);     // 2^73 (e + e^2)
+  const long long corr = ((long long)Y * (e2 >> 13)) >> 25;  // 2^35 Y (e + e^2)
+  const unsigned long long Z = ((unsigned long long)Y << 35) + (unsigned long long)corr;  // 56 bits
   return from_bits(((Z + 4) >> 3) + ((unsigned long long)top << 32));
 }
 

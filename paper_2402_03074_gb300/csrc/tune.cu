@@ -4,7 +4,8 @@
 // work against balance and latency hiding: taller chunks waste fewer ring rows, narrower
 // bands more ring columns and lanes, the tile count sets how evenly the blocks fill the SMs,
 // and the block width (64, 96, 128 or 192 columns) sets the rows of a tile (geometry.h), the
-// resident warps per SM and the idle lanes of a band.  The autotuner times one stage launch of a problem for each candidate shape
+// resident warps per SM and the idle lanes of a band.  The autotuner times one stage launch of a
+// problem for each candidate shape
 // (block width x band count x chunk height) on a scratch copy of the caller's moments (with
 // dt = 0, so the copy does not evolve), times the closest few again over whole three-stage
 // sequences, and keeps the fastest in a process-wide table keyed by (equation,

@@ -72,3 +72,14 @@ def test_every_width_and_chunk_height(tmp_path, eq, ch):
                 np.testing.assert_array_equal(_check(eq, ch, nx, ny, 2, 1), ref)
     finally:
         entry(0, 0)
+
+
+def test_an_overflowed_sound_speed_stays_infinite():
+    """gamma (gamma - 1) e / rho beyond the double range at finite, admissible averages (a uniform
+    state at rest, linear weights, dt = 0): the output's wave speeds are infinite, not lost."""
+    _, hp = problems(2, "euler", 9, 7, characteristic=0, weights=2)
+    U = np.zeros((4, 3, 7, 9))
+    U[0, 0], U[3, 0] = 1e-10, 1e300
+    out, _, speeds, status = gpu_stage(hp, 1, U, U, np.zeros((4, 2, 7, 9)), (1.0, 1.0), 0.0)
+    assert status == 0 and np.array_equal(out[:, 0], U[:, 0])
+    assert np.isposinf(speeds).all()
