@@ -11,8 +11,6 @@
 // status); one thread per solve advances them at the start of each step, so each solve
 // steps with its own dt.  The work lists live in device memory: admission and retirement
 // rewrite them between steps and the captured step graph stays valid.
-#include <vector>
-
 #include "batch.h"
 #include "stage1d_lanes64.cuh"
 #include "stage2d_item.cuh"
@@ -270,23 +268,21 @@ void batch_geometry(int nx, int ny, int rows, int* bands, int* wout, int* chunks
   *chunks = (ny + rows - 1) / rows;
 }
 
-static int sm_count() {
+int batch_sms() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) == cudaSuccess)
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
   return n > 0 ? n : 1;
 }
 
-int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots) {
-  std::vector<int> bands(n), warps(n);
+int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots, int sms,
+                    int* bands, int* warps) {
   for (int s = 0; s < n; ++s) {
     int wout, chunks;
     batch_geometry(nx[s], ny[s], 1, &bands[s], &wout, &chunks);
     warps[s] = (wout + 2 + 31) / 32;
   }
-  const int sms = sm_count();
-  return batch_rows64(bands.data(), warps.data(), ny, n, kBatchBX, slots,
-                      slots > sms ? slots / sms : 1, mixed);
+  return batch_rows64(bands, warps, ny, n, kBatchBX, slots, slots > sms ? slots / sms : 1, mixed);
 }
 
 }  // namespace hw

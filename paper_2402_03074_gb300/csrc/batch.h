@@ -48,8 +48,12 @@ struct BatchDt {
 int batch_class(int equation, int characteristic, int mixed, int dim = 2);
 // bands of at most kBatchBX - 2 columns and row chunks of `rows` rows
 void batch_geometry(int nx, int ny, int rows, int* bands, int* wout, int* chunks);
-// rows per item for the 2D solves of one class (n grids) on `slots` resident blocks
-int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots);
+// SMs of the current device
+int batch_sms();
+// rows per item for the 2D solves of one class (n grids) on `slots` resident blocks of `sms` SMs;
+// bands and warps: the caller's scratch of n entries each (nothing is allocated)
+int batch_item_rows(const int* nx, const int* ny, int n, bool mixed, int slots, int sms,
+                    int* bands, int* warps);
 void batch_geometry1d(int nx, int* blocks);
 int batch_slots(int cls);  // resident blocks of the class's persistent launch
 cudaError_t launch_batch_dt(BatchDt* d, BatchCtl* ctl, int nctl, int cap, cudaStream_t st);

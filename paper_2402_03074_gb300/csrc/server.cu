@@ -164,10 +164,13 @@ static int rebuild_lists(Server* S, cudaStream_t st, unsigned* classes) {
     cy[cls].push_back(p->ny);
   }
   int rows_of[kBatchClasses];
+  const int sms = batch_sms();
+  std::vector<int> bands(S->live.size()), warps(S->live.size());
   for (int c = 0; c < kBatchClasses; ++c)
     rows_of[c] = cx[c].empty() ? S->rows
                                : batch_item_rows(cx[c].data(), cy[c].data(), (int)cx[c].size(),
-                                                 (c & 1) != 0, batch_slots(c));
+                                                 (c & 1) != 0, batch_slots(c), sms, bands.data(),
+                                                 warps.data());
   int n = 0, nall = 0;
   *classes = 0;
   for (Request* r : S->live) {

@@ -102,6 +102,7 @@ struct StaticSetup {
   StaticScratch* ptr = nullptr;
   int slots[kBatchClasses] = {};
   size_t local[kBatchClasses] = {};
+  int sms = 1;
 };
 static std::mutex g_static_mu;
 static StaticSetup g_static[64];
@@ -143,6 +144,7 @@ static int static_device_setup(int dev) {
   void* p = nullptr;
   if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return HWENO_ERR_CUDA;
   S.ptr = static_cast<StaticScratch*>(p);
+  S.sms = batch_sms();
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = static_class_setup<EQ_ADV, false, double>(&S.slots[0], &S.local[0]);
   if (e == cudaSuccess) e = static_class_setup<EQ_ADV, false, float>(&S.slots[1], &S.local[1]);
@@ -213,11 +215,12 @@ extern "C" int hweno_stage_batch_static(int n, const hweno_problem* problems, in
   std::memset(&host, 0, sizeof(host));
   const bool mixed = p0.precision == HWENO_MIXED32;
   int nxs[HWENO_STATIC_BATCH_MAX], nys[HWENO_STATIC_BATCH_MAX];
+  int bands[HWENO_STATIC_BATCH_MAX], warps[HWENO_STATIC_BATCH_MAX];
   for (int s = 0; s < n; ++s) {
     nxs[s] = problems[s].nx;
     nys[s] = problems[s].ny;
   }
-  const int rows = batch_item_rows(nxs, nys, n, mixed, D.slots[cls]);
+  const int rows = batch_item_rows(nxs, nys, n, mixed, D.slots[cls], D.sms, bands, warps);
   int items = 0;
   for (int s = 0; s < n; ++s) {
     StaticItem& it = host.item[s];
