@@ -174,6 +174,17 @@ inline Tile64 default_tile64(int nx, int ny, int sms, const int* bx, const int* 
   return best;
 }
 
+// Whether a shape of the tuning table (launch.h, TileShape) leaves the tile to the rule above: no
+// width and nothing fixed, or the autotuner's entry for it, {0, 0, kDefaultWidth2D}.  Any other
+// shape with a width is of that width, with the band and row geometry of geom2d where these are
+// not fixed (the same bits, another kernel: 240^2 Euler FP64 in 96 columns, {-1, -1, 96}, takes
+// 1.4 times the rule's 32).
+constexpr int kDefaultWidth2D = 96;
+inline bool takes_default_tile(int rows, int bands, int width) {
+  if (width == 0) return (rows == 0 || rows == -1) && bands <= 0;
+  return width == kDefaultWidth2D && rows == 0 && bands == 0;
+}
+
 // Rows per item of a batched 2D class in tiles of bx columns (bands[s] bands of warps[s] warps
 // per row, ny[s] rows), whose persistent launch has `slots` resident blocks: the rows of least
 // waves x item time (per_sm blocks sharing an SM), the smallest (the most items) among equals.

@@ -64,15 +64,13 @@ __device__ __forceinline__ void dt_update(DevScal* s, double inv_dx, double inv_
 struct TileShape {
   int rows = 0;
   int bands = 0;
-  // block width: 2D 32, 64, 96, 128 or 192 columns (0 = the default); 1D 0 = the default rule,
-  // else 32, 64 or 128 threads.  1D threads per cell (0 or 1: one thread per cell; 4: one lane per
-  // characteristic field, 1D Euler with the characteristic decomposition)
+  // block width: 2D 32, 64, 96, 128 or 192 columns (0, or 96 with rows = bands = 0: the tile chosen
+  // for the grid, geometry.h); 1D 0 = the default rule, else 32, 64 or 128 threads.  1D threads per
+  // cell (0 or 1: one thread per cell; 4: four lanes per cell, in FP64 for every equation, in
+  // FP32-bulk for Euler with the characteristic decomposition)
   int width = 0;
   int lanes = 0;
 };
-// Default block width of the 2D single-solve launch: 96 columns; with the default geometry the
-// tile is then chosen for the grid (geometry.h).
-constexpr int kDefaultWidth2D = 96;
 // Tuning table keyed by (equation, characteristic, precision, nx, ny); all zero = not tuned.
 TileShape tuning_shape(int eq, int characteristic, int mixed, int nx, int ny);
 void tuning_set_shape(int eq, int characteristic, int mixed, int nx, int ny, TileShape t);

@@ -17,7 +17,7 @@ cudaError_t launch_stage2d(int eq, bool characteristic, bool mixed, const KProbl
   if (t.rows == 0 && t.bands == 0 && t.width == 0)
     t = tuning_shape(eq, ch ? 1 : 0, mixed ? 1 : 0, P.nx, P.ny);
   int w = t.width > 0 ? t.width : kDefaultWidth2D;
-  if (w == kDefaultWidth2D && t.rows >= -1 && t.rows <= 0 && t.bands <= 0) {
+  if (takes_default_tile(t.rows, t.bands, t.width)) {
     // the default: the tile width and chunk height of least time for the grid (geometry.h)
     static const int bx[3] = {32, 64, 96};
     int slots[3], sms = 0, dev = 0;

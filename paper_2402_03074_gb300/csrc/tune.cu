@@ -5,7 +5,7 @@
 // bands more ring columns and lanes, the tile count sets how evenly the blocks fill the SMs,
 // and the block width (64, 96, 128 or 192 columns) sets the rows of a tile (geometry.h), the
 // resident warps per SM and the idle lanes of a band.  The autotuner times one stage launch of a
-// problem for each candidate shape
+// problem in the tile that a grid without an entry takes and in each candidate shape
 // (block width x band count x chunk height) on a scratch copy of the caller's moments (with
 // dt = 0, so the copy does not evolve), times the closest few again over whole three-stage
 // sequences, and keeps the fastest in a process-wide table keyed by (equation,
@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "../../include/hweno.h"
+#include "geometry.h"
 #include "launch.h"
 #include "server.h"
 
@@ -140,7 +141,8 @@ int hweno_autotune(hweno_engine* e, const hweno_problem* p, const double* host, 
     if (rc) engine_set_error(e, "autotune launch failed");
     return rc;
   }
-  // candidates: block widths (128, 96, 64 and 192 threads) x band counts (0 = the default bands; then
+  // candidates: the tile a grid without an entry takes (so that tuning never settles for a slower
+  // one); then block widths (128, 96, 64 and 192 columns) x band counts (0 = the default bands; then
   // 1.25, 1.5 and 2 times as many as the widest bands of that width) x chunk heights (0 = one
   // wave over the resident slots).  Screened on stage 1 (the fastest of three launches after
   // one untimed); the finalists -- at most four, within 3 % of the fastest -- are then timed
@@ -176,6 +178,13 @@ int hweno_autotune(hweno_engine* e, const hweno_problem* p, const double* host, 
     return tmin;
   };
   std::vector<std::pair<float, TileShape>> screened;
+  {
+    TileShape t;
+    t.width = kDefaultWidth2D;  // rows = bands = 0: takes_default_tile
+    const float ms = time_shape(t, 1, 1, 4);
+    if (ms < 0.f) rc = HWENO_ERR_CUDA;
+    else screened.push_back({ms, t});
+  }
   for (int wi = 0; wi < kWidths && rc == HWENO_OK; ++wi) {
     const int bw = widths[wi];
     const int bmin = (p->nx + bw - 3) / (bw - 2);
@@ -226,12 +235,8 @@ int hweno_autotune(hweno_engine* e, const hweno_problem* p, const double* host, 
     engine_set_error(e, "autotune launch failed");
     return rc;
   }
-  TileShape keep;
-  keep.rows = best.rows > 0 ? best.rows : -1;
-  keep.bands = best.bands > 0 ? best.bands : -1;
-  keep.width = best.width;
   tuning_set_shape(p->equation, p->equation == HWENO_EULER ? p->characteristic : 0,
-                   p->precision == HWENO_MIXED32, p->nx, p->ny, keep);
+                   p->precision == HWENO_MIXED32, p->nx, p->ny, best);
   if (best_rows) *best_rows = best.rows > 0 ? best.rows : 0;
   if (best_bands) *best_bands = best.bands > 0 ? best.bands : 0;
   if (best_ms) *best_ms = best_t;
