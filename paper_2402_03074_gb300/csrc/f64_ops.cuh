@@ -39,16 +39,18 @@ __device__ __forceinline__ Ops make_ops(const double* tab, int k) {
   return o;
 }
 
-// 1/x of a normal double with exponent field in [1, 2044], from the hardware's 20-bit reciprocal,
-// by a third-order step.  On integers (rcp64.h) where many warps share the FP64 unit:
-// about 30 integer instructions instead of three FP64 operations, 1/40 of a 2D Euler cell's time
-// (2048^2 step 56.5 -> 55.1 ms, 768^2 component-wise 5.50 -> 5.30 ms).
+// 1/x of a normal double with exponent field in [1, 2044], from the hardware's reciprocal of about
+// 20 bits (its residual e = 1 - x y is below 2^-19.9, measured over all the leading words it looks
+// at), by the first terms of the geometric series 1/(1 - e) = 1 + e + e^2 + ..  On integers (rcp64.h),
+// within 0.51 ulp, where many warps share the FP64 unit: about 30 integer instructions instead of
+// three FP64 operations, 1/40 of a 2D Euler cell's time (2048^2 step 56.5 -> 55.1 ms, 768^2
+// component-wise 5.50 -> 5.30 ms).
 __device__ __forceinline__ double rcp_in_range(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   return rcp64_refine(x, y);
 }
-// The same in three FMAs, for the 1D kernels' lone warps and the FP32-bulk kernels.
+// The same in three FMAs, within 0.51 ulp, for the 1D kernels' lone warps and the FP32-bulk kernels.
 __device__ __forceinline__ double rcp_in_range(const Ops& o, double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -66,16 +68,34 @@ __device__ __forceinline__ double rcp_any(const Ops& o, double x) {
   return rcp_applies(x) ? rcp_in_range(o, x) : 1.0 / x;
 }
 
-// 1/sqrt(x): the hardware's 20-bit value y refined by one third-order step y (1 + e/2 + 3 e^2/8),
-// e = 1 - x y^2 (the new residual is below 2^-59); the library's where x is near the ends of the
-// range or not positive.  half and c38: 1/2 and 3/8.
-__device__ __forceinline__ double rsqrt_any(const Ops& o, double x, double half, double c38) {
+// 1/sqrt(x): the hardware's 20-bit value y refined by the first three terms of the binomial series
+// of (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + .., e = 1 - x y^2 (the next, 5 e^3/16, is below 2^-58);
+// the library's where x is near the ends of the range or not positive.  Within 1 ulp (measured
+// 0.99; the rounding of x y shows in e).  half and c38: 1/2 and 3/8.
+__device__ __forceinline__ bool root_applies(double x) {
   const int eb = __double2hiint(x) >> 20;
-  if (eb < 64 || eb > 1983) return rsqrt(x);
+  return eb >= 64 && eb <= 1983;
+}
+__device__ __forceinline__ double rsqrt_any(const Ops& o, double x, double half, double c38) {
+  if (!root_applies(x)) return rsqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-o.mul(x, y), y, o.one);
   return fma(o.mul(y, e), fma(c38, e, half), y);
+}
+
+// sqrt(x): g = x y refined by the same series, then by one step of Newton's iteration with the
+// exact residual, s + (x - s^2) y/2 (y/2 by its exponent field): within 0.501 ulp (the library's bits
+// in 2^20 values of the whole range), for the wave speeds that set alpha and dt.  One FP64
+// operation more than x rsqrt_any(x), which would be within 2 ulp.
+__device__ __forceinline__ double sqrt_any(const Ops& o, double x, double half, double c38) {
+  if (!root_applies(x)) return sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = o.mul(x, y), e = fma(-g, y, o.one);
+  const double s = fma(o.mul(g, e), fma(c38, e, half), g);
+  const double yh = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));
+  return fma(fma(-s, s, x), yh, s);
 }
 
 }  // namespace hw

@@ -31,8 +31,10 @@ HW_RCP64 double from_bits(unsigned long long b) {
 }
 
 // 1/x of a normal double with exponent field in [1, 2044] from y, its reciprocal to about 20 bits
-// (the low word of y is zero, |1 - x y| < 2^-18): y (1 + e + e^2), e = 1 - x y, the first terms of
-// the geometric series of 1/(1 - e), on the mantissas.
+// (the low word of y is zero, |1 - x y| < 2^-19, and y is in the binade of 1/x or, for x next to a
+// power of two, at its lower end): y (1 + e + e^2), e = 1 - x y, the first terms of the geometric
+// series of 1/(1 - e), on the mantissas.  Within 0.58 ulp: a rounding, e^3 < 2^-57 (1/16 ulp) and
+// the truncation of e (1/128 ulp).
 HW_RCP64 double rcp64_refine(double x, double y) {
   const unsigned long long bx = bits_of(x);
   const unsigned hy = (unsigned)(bits_of(y) >> 32);

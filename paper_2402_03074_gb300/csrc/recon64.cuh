@@ -376,8 +376,7 @@ __device__ __forceinline__ bool speeds(const Ops& o, const double (&u)[4], doubl
   const double vx = o.mul(u[1], ir), vy = o.mul(u[2], ir);
   const double e = fma(-K(HALF), fma(u[1], vx, o.mul(u[2], vy)), u[3]);
   const double c2 = o.mul(o.mul(o.mul(K(GAM), K(GM1)), e), ir);
-  // a root of 0 or of an overflowed value is that value
-  const double c = c2 > 0.0 && finite_bits(c2) ? o.mul(c2, rsqrt_any(o, c2, K(HALF), K(RS2))) : c2;
+  const double c = sqrt_any(o, c2, K(HALF), K(RS2));
   s0 = o.add(fabs(vx), c);
   s1 = o.add(fabs(vy), c);
   return u[0] > 0.0 && e > 0.0 && finite_bits(e);

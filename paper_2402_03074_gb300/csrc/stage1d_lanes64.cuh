@@ -142,7 +142,7 @@ struct Frame1 {
     const double rc = rsqrt_any(o, c2, K(HALF), K(RS2));
     cs = o.mul(c2, rc);
     H = o.mul(o.add(U2, p), ir);
-    b1h = -o.mul(o.mul(K(HGM1), rc), rc);
+    b1h = -o.mul(K(HGM1), rcp_any(o, c2));  // rounded once less than from rc twice
     hic = o.mul(K(HALF), rc);
   }
   __device__ __forceinline__ void row(const Ops& o, double sf, double sh, double df, double& l0,
@@ -237,7 +237,7 @@ __device__ __forceinline__ double speed64(const Ops& o, const double (&ua)[3], b
   const double e = fma(-o.mul(K(HALF), ua[1]), vn, ua[2]);  // internal energy density
   const double c2 = o.mul(o.mul(o.mul(K(GAM), K(GM1)), e), ir);
   ok &= ua[0] > 0.0 && e > 0.0 && finite_bits(e);
-  return c2 > 0.0 ? fma(c2, rsqrt_any(o, c2, K(HALF), K(RS2)), fabs(vn)) : fabs(vn);
+  return o.add(fabs(vn), sqrt_any(o, c2, K(HALF), K(RS2)));
 }
 
 }  // namespace l64
