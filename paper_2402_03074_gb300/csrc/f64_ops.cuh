@@ -28,10 +28,14 @@ struct Ops {
   __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, nz); }
 };
 
-// The operations on the table `tab` (entries One and MinusZero hold 1 and -0).  k is the stage
-// number, at most 3: k >> 2 is 0 for every thread, which the compiler cannot prove.
+// The operations on the table `tab` (entries One and MinusZero hold 1 and -0), which a barrier has
+// made visible to the thread.  k is the stage number, at most 3: k >> 2 is 0 for every thread,
+// which the compiler cannot prove.
 template <int One, int MinusZero>
 __device__ __forceinline__ Ops make_ops(const double* tab, int k) {
+  // the reads below are volatile and follow this statement, which no memory access crosses: none
+  // moves above the barrier after the table's filling
+  asm volatile("" : : : "memory");
   Ops o;
   o.tab = (unsigned)__cvta_generic_to_shared(tab) + (unsigned)((k >> 2) * (int)threadIdx.x);
   o.one = o.k<One>();
