@@ -1,6 +1,6 @@
 // stage1d_item.cuh -- one block of the fused 1D HWENO-U stage (Sec. 2.1, Eq. 2.3, 2.4, 2.12,
-// 2.13), shared by the single-solve kernel (stage1d.cu) and the batched persistent kernel
-// (batch.cu).
+// 2.13) in FP32-bulk arithmetic, shared by the single-solve kernels (stage1d.cu) and the batched
+// persistent kernel (batch.cu); the FP64 block is in stage1d_lanes64.cuh.
 //
 // One thread per reconstructed cell.  Block blk of BW threads reconstructs cells
 // [i0-1, i0+BW-1), i0 = blk (BW-2), and updates the BW-2 cells [i0, i0+BW-2): every cell is
@@ -12,7 +12,7 @@
 namespace hw {
 
 // Where a 1D item's stage input, base state U^n, V-hat, output and scalars live: device
-// memory through the stage's pointers (the per-stage launches); stage1d_cluster.cuh has the
+// memory through the stage's pointers (the per-stage launches); Cluster1D in stage1d.cu is the
 // shared-memory counterpart of a solve resident in a thread-block cluster.
 struct Global1D {
   static constexpr bool kTabulated = false;  // the window is filled by the generic loop
@@ -40,6 +40,7 @@ struct Global1D {
 
 template <int EQ, bool CHAR, typename R, int BW, class IO>
 __device__ __forceinline__ void stage1d_item_io(const KProblem& P, const IO& io, int blk) {
+  static_assert(sizeof(R) == sizeof(float), "the FP64 block: stage1d_lanes64.cuh");
   constexpr int NC = (EQ == EQ_EULER) ? 3 : 1;
   constexpr int NM = 2;
   const int nx = P.nx;
@@ -154,8 +155,7 @@ __device__ __forceinline__ void stage1d_item_io(const KProblem& P, const IO& io,
       const R F1 = -(fr - fl) * idx;
       const R vol = R(1.0 / 12.0) * (fp[0][c] + fp[3][c]) + R(5.0 / 12.0) * (fp[1][c] + fp[2][c]);
       const R F2 = (vol - R(0.5) * (fl + fr)) * idx;
-      const double own_u = (sizeof(R) == sizeof(double)) ? to_f64(win[c * NM][t + 1])
-                                                          : io.in(c * NM, i);
+      const double own_u = io.in(c * NM, i);
       const double own_v = to_f64(vh[c]);
       double base_u, base_v;
       if (k == 1) {
@@ -219,6 +219,7 @@ __device__ __forceinline__ void stage1d_item_io(const KProblem& P, const IO& io,
 // short to fill the GPU with one thread per cell.  Every lane of a warp runs every shuffle.
 template <typename R, int BW, class IO>
 __device__ __forceinline__ void stage1d_fields_item_io(const KProblem& P, const IO& io, int blk) {
+  static_assert(sizeof(R) == sizeof(float), "the FP64 block: stage1d_lanes64.cuh");
   constexpr int NC = 3, NM = 2, G = BW / 4;
   const int nx = P.nx;
   const int t = threadIdx.x, q = t >> 2, f = t & 3;
@@ -298,8 +299,7 @@ __device__ __forceinline__ void stage1d_fields_item_io(const KProblem& P, const 
     const R F1 = -(fR - fL) * idx;
     const R vol = R(1.0 / 12.0) * (fp[0][f] + fp[3][f]) + R(5.0 / 12.0) * (fp[1][f] + fp[2][f]);
     const R F2 = (vol - R(0.5) * (fL + fR)) * idx;
-    const double own_u = (sizeof(R) == sizeof(double)) ? to_f64(win[f * NM][q + 1])
-                                                        : io.in(f * NM, i);
+    const double own_u = io.in(f * NM, i);
     const double own_v = to_f64(vh[f]);
     double base_u, base_v;
     if (k == 1) {

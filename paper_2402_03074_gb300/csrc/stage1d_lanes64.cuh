@@ -31,7 +31,6 @@ enum : int {
   kT, kB,                      // term of beta_0: KB (c_{l+1} + KT c_{l+3})^2
   kX1, kX2, kX3, kX4,          // point l: u = mean + X1 C1 + X2 C2 + X3 C3 + X4 C4
   kSF, kSH, kDF,               // row l of L: factors of b1h and of 1/(2c), constant
-  kSign,                       // the sign of alpha u beside the flux in the trace of point l
   kLane
 };
 constexpr double R5 = 0.22360679774997896964;  // sqrt(5)/10
@@ -48,8 +47,7 @@ static __constant__ double lane_constants[kLane][4] = {
     {1.0 / 16.0 - 1.0 / 80.0, 0.0025 - 1.0 / 80.0, 0.0025 - 1.0 / 80.0, 1.0 / 16.0 - 1.0 / 80.0},
     {1.0, -2.0, 1.0, 1.0},
     {-1.0, 0.0, 1.0, 1.0},
-    {0.0, 1.0, 0.0, 0.0},
-    {-1.0, 1.0, 1.0, 1.0}};
+    {0.0, 1.0, 0.0, 0.0}};
 
 #define HW_L64_CONSTANTS(X)                                                                   \
   X(ONE, 1.0) X(MZERO, -0.0) X(TAU, 2.25) X(V1, 1.0 / 12.0) X(V3, 1.0 / 80.0) X(HALF, 0.5)    \
