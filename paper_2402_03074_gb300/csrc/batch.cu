@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(BW) batch1d_stage_kernel(const BatchSolve* bs,
     S.status = &B.sc->status;
     S.active = &B.sc->active;
     S.k = k;
-    if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, B.P);
-    thread_item1d<EQ, CHAR, R, BW>(B.P, S, item - B.item_base, tab);
+    if constexpr (sizeof(R) == sizeof(double)) l64::fill_table<BW>(tab, B.P);
+    thread_item1d<EQ, CHAR, R, BW>(B.P, S, item - B.item_base, tab, l64::TableFilled{});
   }
 }
 

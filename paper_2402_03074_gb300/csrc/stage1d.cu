@@ -39,18 +39,22 @@ template <int EQ, bool CHAR, typename R, int BW>
 __global__ void __launch_bounds__(BW) stage1d_kernel(KProblem P, KStage S) {
   if (S.active && *S.active == 0) return;
   __shared__ double tab[l64::kTable];
-  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, P);
-  thread_item1d<EQ, CHAR, R, BW>(P, S, blockIdx.x, tab);
+  l64::TableFill<BW> table;
+  if constexpr (sizeof(R) == sizeof(double)) table.load();
+  thread_item1d<EQ, CHAR, R, BW>(P, S, blockIdx.x, tab, table);
 }
 
 // classes with a layout of four lanes per cell
 template <int EQ, bool CHAR, typename R>
 constexpr bool kLanes1D = sizeof(R) == sizeof(double) || (EQ == EQ_EULER && CHAR);
 
-// one block of the four-lanes layout; tab: the FP64 table of constants, filled by the block
-template <int EQ, bool CHAR, typename R, int BW, class IO>
-__device__ __forceinline__ void lanes_item(const KProblem& P, const IO& io, int blk, double* tab) {
-  if constexpr (sizeof(R) == sizeof(double)) stage1d_lanes64_item_io<EQ, CHAR, BW>(P, io, blk, tab);
+// one block of the four-lanes layout; tab: the FP64 table of constants, stored by `table` (or filled
+// by the block before the call)
+template <int EQ, bool CHAR, typename R, int BW, class IO, class Fill>
+__device__ __forceinline__ void lanes_item(const KProblem& P, const IO& io, int blk, double* tab,
+                                           const Fill& table) {
+  if constexpr (sizeof(R) == sizeof(double))
+    stage1d_lanes64_item_io<EQ, CHAR, BW>(P, io, blk, tab, table);
   else stage1d_fields_item_io<R, BW>(P, io, blk);
 }
 
@@ -58,9 +62,10 @@ template <int EQ, bool CHAR, typename R, int BW>
 __global__ void __launch_bounds__(BW) stage1d_lanes_kernel(KProblem P, KStage S) {
   if (S.active && *S.active == 0) return;
   __shared__ double tab[l64::kTable];
-  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, P);
+  l64::TableFill<BW> table;
+  if constexpr (sizeof(R) == sizeof(double)) table.load();
   const Global1D io{S, P.nx};
-  lanes_item<EQ, CHAR, R, BW>(P, io, blockIdx.x, tab);
+  lanes_item<EQ, CHAR, R, BW>(P, io, blockIdx.x, tab, table);
 }
 
 template <int EQ, bool CHAR, typename R>
@@ -110,7 +115,7 @@ template <int EQ, bool CHAR, typename R, int BW, bool LANES>
 __global__ void __launch_bounds__(BW) step1d_coop_kernel(Step1D A, int nsteps, int items) {
   cg::grid_group grid = cg::this_grid();
   __shared__ double tab[l64::kTable];
-  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(tab, A.P);
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table<BW>(tab, A.P);
   volatile int* active = &A.sc->active;
 #pragma unroll 1
   for (int s = 0; s < nsteps; ++s) {
@@ -132,8 +137,9 @@ __global__ void __launch_bounds__(BW) step1d_coop_kernel(Step1D A, int nsteps, i
       S.k = k;
 #pragma unroll 1
       for (int it = blockIdx.x; it < items; it += gridDim.x) {
-        if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, Global1D{S, A.P.nx}, it, tab);
-        else thread_item1d<EQ, CHAR, R, BW>(A.P, S, it, tab);
+        const l64::TableFilled filled;
+        if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, Global1D{S, A.P.nx}, it, tab, filled);
+        else thread_item1d<EQ, CHAR, R, BW>(A.P, S, it, tab, filled);
       }
       grid.sync();
     }
@@ -247,7 +253,7 @@ __global__ void __launch_bounds__(kClusterBW<LANES>) step1d_cluster_kernel(Step1
   __shared__ unsigned bad[4][1];  // [k]: this CTA's non-physical flag of stage k
   __shared__ DevScal scl;         // the solve's scalars (every CTA holds the same values)
   __shared__ double ctab[l64::kTable];
-  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table(ctab, A.P);
+  if constexpr (sizeof(R) == sizeof(double)) l64::fill_table<BW>(ctab, A.P);
   const int rank = (int)cl.block_rank(), nb = (int)cl.num_blocks();
   const int nx = A.P.nx, i0 = rank * W, t = threadIdx.x;
   for (int q = t; q < NA * W; q += BW) {
@@ -296,7 +302,7 @@ __global__ void __launch_bounds__(kClusterBW<LANES>) step1d_cluster_kernel(Step1
       Cluster1D<NA, W, SL, R> io{st, vhs, &amax[k][0], &bad[k][0], &tab, k - 1, k % 3, k, i0,
                                  scl.dt, scl.alpha[k - 1][0]};
       if (t == 0) bad[k][0] = 0u;
-      if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, io, rank, ctab);
+      if constexpr (LANES) lanes_item<EQ, CHAR, R, BW>(A.P, io, rank, ctab, l64::TableFilled{});
       else stage1d_item_io<EQ, CHAR, R, BW>(A.P, io, rank);
     }
   }
