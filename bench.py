@@ -46,16 +46,16 @@ FP32_PEAK_TFLOPS_FALLBACK = 74.2
 # FP64 arithmetic the fused 2D Euler characteristic kernel executes per cell-stage, from the
 # ncu thread-instruction counts of one 2048^2 launch in its default geometry (96 x 2 tiles, 22
 # bands of 94 columns in 152 segments of 297 band-rows;
-# profiles/stage2d_euler_2048_instruction_counts.md) per updated cell less the 2.5 % of
+# profiles/instruction_counts.md) per updated cell less the 2.5 % of
 # redundant ring-cell reconstruction: operations (DFMA + DMUL + DADD) of stage 1, the timed
-# launch, 2370 -> 2312 (2335 in stages 2 and 3).  The FP64
+# launch, 2371 -> 2313 (2337 in stages 2 and 3).  The FP64
 # pipe executes one such operation per lane per clock, so its operation rate is half the FMA
 # flop rate.
-FP64_OPS_PER_CELL_STAGE = 2312.0
+FP64_OPS_PER_CELL_STAGE = 2313.0
 # DRAM bytes read + written by the same launch (ncu)
-FP64_STAGE_DRAM_BYTES = 499.4e6 + 661.5e6
+FP64_STAGE_DRAM_BYTES = 499.4e6 + 662.5e6
 # FP64 pipe utilisation of the same launch (% of peak sustained, active cycles)
-FP64_PIPE_UTIL_NCU = 0.929
+FP64_PIPE_UTIL_NCU = 0.930
 # FP32-bulk kernel (same workload, ncu): FP64 arithmetic operations per cell-stage (832 per
 # updated cell in its default geometry, 96 x 2 tiles, less 2.5 % ring redundancy; stages 2 and
 # 3), FP32 flops, and the DRAM bytes of a stage 1 launch
@@ -724,10 +724,7 @@ def tubes_1d(H, I, eng_factory, tubes, n, t_end, autotune=True):
             "speedup": el_plain / el_b, "max_rel_diff_batched_vs_plain": diff,
             "tube0_batched_vs_plain_same_layout": same_layout,
             "diff_note": "the batched path and the default single-solve layout run the same "
-                         "code (tube 0: bitwise equal); the lanes-per-field layout rounds "
-                         "differently, and over the thousands of steps of a shock tube the "
-                         "shocks amplify that to the level a 1-ulp change of the data "
-                         "reaches (1e-3 of the component scale)",
+                         "operations (bitwise equal in FP64, whatever the threads per cell)",
             "same_steps": steps_b == steps}
 
 

@@ -8,10 +8,10 @@
 namespace hw {
 
 // Block width of the batched stage kernels: the 1D classes 128 threads, the 2D classes tiles of 64
-// columns x 3 rows (against one row at a time in 128-thread blocks, which hold only four warps
-// per SM in FP64: a batch of eight FP64 solves of 200 x 184 to 284 x 261 cells, one step, 9.00 ->
-// 7.58 ms; a served mix of six grids of 128^2 to 352^2 cells, a third of them FP32-bulk, 114 ->
-// 95.5 ms with the FP64 classes in tiles).
+// columns by 4 rows in FP64 and 3 in FP32-bulk (against one row at a time in 128-thread blocks, which
+// hold only four warps per SM in FP64, and FP64 tiles of 3 rows: a batch of eight FP64 solves of
+// 200 x 184 to 284 x 261 cells, one step, 9.00, 7.58 and now 6.80 ms; a served mix of six grids of
+// 128^2 to 352^2 cells, a third of them FP32-bulk, 114, 95.5 and now 85.4 ms).
 constexpr int kBatchBW = 128;
 constexpr int kBatchBX = 64;
 constexpr int kBatchClasses = 16;  // {2D, 1D} x {advection, Burgers, Euler comp.-wise,

@@ -3,11 +3,10 @@
 // single-solve launch (stage2d.cu), the batched launches (batch.cu, static_batch.cu) and the
 // serving loop (server.cu).
 //
-// A block of bw threads covers a band of at most bw - 2 output columns plus one ring column
-// on each side, and sweeps a chunk of rows (one ring row above and below).  The time of a
-// launch is set by its waves of items over the resident block slots and by the rows of an
-// item: a block's row sweep is bound by the latency of its own instruction stream, so a block
-// alone on an SM is not faster than one of two sharing it.
+// A block of bw columns (by one to eight rows) of threads covers a band of at most bw - 2 output
+// columns plus one ring column on each side, and sweeps a chunk of rows (one ring row above and
+// below), several rows at a time.  The time of a launch is set by its waves of items over the
+// resident block slots and by the steps of an item (tile_time64).
 #pragma once
 
 namespace hw {
@@ -19,11 +18,9 @@ inline int band_lanes(int nx, int bands) {
   return bands * 32 * ((w + 2 + 31) / 32);
 }
 
-// Default band count for blocks of bw threads: the widest bands (at most bw - 2 output
-// columns).  With lane_aware (the FP64 kernels, whose two blocks per SM keep the FP64 pipe
-// busy with three active warps each), bands of at most bw - 34 columns when they leave fewer
-// idle lanes (2048 columns: 22 bands of 94 columns in 96 lanes each rather than 17 of 121 in
-// 128).
+// Default band count for blocks of bw columns: the widest bands (at most bw - 2 output columns).
+// With lane_aware, which no launch asks for since the tiles have several rows (the host tests do),
+// bands of at most bw - 34 columns when they leave fewer idle lanes.
 inline int default_bands(int nx, int bw, bool lane_aware) {
   int b = (nx + (bw - 2) - 1) / (bw - 2);
   if (lane_aware && bw > 34) {
@@ -47,13 +44,12 @@ inline void split_bands(int nx, int bands_req, int* bands, int* wout) {
 //  * segments (seg > 0): the bands' rows taken one after another (band-row q = band ny + row)
 //    and cut into `blocks` equal segments of seg band-rows, one per block; a segment that
 //    crosses the end of a band is swept as two (or more) pieces.  When the band count does not
-//    divide the slots, chunks leave slots empty (2048^2 in 94-column bands: 22 x 13 = 286 of
-//    304), while segments fill them (303 blocks of 149 band-rows instead of 158 rows).
-// Fixed rows > 0 give chunks of that height, fixed rows < -1 segments of -rows band-rows; the
-// default (0) takes segments where they cost at least 2 % less than chunks, a piece costing
-// its rows plus about 1.5 rows (its two ring rows of the y pass and the window prologue)
-// (2048^2 FP64: 29.05 ms instead of 29.65 ms per stage; a 0.6 % estimate, as for the
-// FP32-bulk kernel's 17 bands on 456 slots, measured nothing).
+//    divide the slots, chunks leave slots empty (2048^2 in 94-column bands: 22 x 6 = 132 of
+//    152), while segments fill them (152 blocks of 297 band-rows instead of 342 rows).
+// Fixed rows > 0 give chunks of that height, fixed rows < -1 segments of -rows band-rows (the rule
+// for a grid without a tuned shape, default_tile64, fixes one or the other); the default (0), of a
+// stored width, takes segments where they cost at least 2 % less than chunks, a piece costing its
+// rows plus about 1.5 rows (its two ring rows of the y pass and the window prologue).
 struct Geom2D {
   int bands, wout, chunks, rows;
   int seg;     // > 0: segment layout, band-rows per block
@@ -250,9 +246,10 @@ inline int batch_rows64(const int* bands, const int* warps, const int* ny, int n
   }
 }
 
-// Rows per work item for the 2D solves of one batched class (bands[s] bands and ny[s] rows
-// each) whose persistent launch has `slots` resident blocks.  The launch runs
-// ceil(items / slots) waves, a partial last wave costing a whole item time, and an item costs
+// The rule for blocks of one row of threads, which the batched launches no longer are (batch_rows64
+// is theirs; the host tests keep this one): rows per work item for the 2D solves of one batched class
+// (bands[s] bands and ny[s] rows each) whose persistent launch has `slots` resident blocks.  The
+// launch runs ceil(items / slots) waves, a partial last wave costing a whole item time, and an item costs
 // its rows plus about 1.5 rows (its two ring rows of the y pass and the three-row window
 // prologue); the rows minimising waves x (rows + 1.5) give the shortest launch, the smallest
 // such rows (the most items) winning ties.

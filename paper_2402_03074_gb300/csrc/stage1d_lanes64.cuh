@@ -10,13 +10,14 @@
 //    of all fields, its flux and its trace; lane c updates component c;
 //  * scalar laws: lane l forms the coefficient c_{l+1} of p_0 and its term of beta_0, then the
 //    point l.
-// The lanes exchange their parts through shared memory.  A stage is then about 180 FP64
-// instructions of a warp for Euler and 70 for a scalar law, instead of 325 and 110 in the
+// The lanes exchange their parts through shared memory.  A stage is then about 190 FP64
+// instructions of a warp for Euler and 74 for a scalar law, instead of 325 and 110 in the
 // lanes-per-field and one-thread-per-cell layouts before.  The block's largest speed takes two
 // integer reductions (a double maximum over a warp costs 135 clocks per shuffle), divisions and
 // square roots are refined from the hardware's 20-bit values (a double square root costs 1070
-// clocks).  Measured, whole calls: 4000-cell Euler shock tube, 128 steps, 8.70 -> 4.10 ms;
-// 240-cell Euler, 400 steps, 16.9 -> 10.4 ms; 200-cell advection, 334 steps, 5.97 -> 4.45 ms.
+// clocks).  Measured, whole calls: 4000-cell Euler shock tube, 128 steps, 8.70 -> 4.01 ms;
+// 240-cell Euler, 400 steps, 16.9 -> 10.6 ms; 200-cell advection, 334 steps, 5.97 -> 4.45 ms.
+// The halves of the Lax-Friedrichs flux are formed as in stage2d_tile64.cuh.
 #pragma once
 #include "f64_ops.cuh"
 #include "hweno_device.cuh"

@@ -1,5 +1,5 @@
 // stage2d.cu -- single-solve launch of the fused 2D HWENO-U stage: the dispatch over block
-// widths (the tuning table's or the class default) and the 128-thread instantiations; the
+// widths (the tuning table's or the tile chosen for the grid) and the 128-column instantiations; the
 // kernel and its launch are in stage2d_impl.cuh, the work item in stage2d_item.cuh.
 #include "stage2d_impl.cuh"
 

@@ -1,7 +1,7 @@
 // stage2d_impl.cuh -- the single-solve 2D stage kernel and its launch for one block width,
-// instantiated per width in stage2d.cu (128 threads), stage2d_w96.cu, stage2d_w64.cu and
-// stage2d_w192.cu so the widths compile in parallel; the dispatch over widths and classes is
-// in stage2d.cu.
+// instantiated per width in stage2d.cu (128 columns), stage2d_w32.cu, stage2d_w64.cu,
+// stage2d_w96.cu and stage2d_w192.cu so the widths compile in parallel; the dispatch over widths
+// and classes is in stage2d.cu.
 #pragma once
 #include "geometry.h"
 #include "launch.h"

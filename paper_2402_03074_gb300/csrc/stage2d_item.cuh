@@ -1,16 +1,18 @@
 // stage2d_item.cuh -- one work item of the fused 2D HWENO-U stage (Sec. 2.2, Eq. 2.16, 2.23,
-// 2.13), shared by the single-solve kernel (stage2d.cu) and the batched persistent kernel
-// (batch.cu).
+// 2.13), shared by the single-solve kernel (stage2d_impl.cuh) and the batched ones (batch.cu,
+// static_batch.cu): the tile of a class, and the item in FP32-bulk arithmetic (the FP64 item:
+// stage2d_tile64.cuh).
 //
-// Decomposition: a block owns a band of wout <= BW-2 output columns and a chunk of output
-// rows [j0, j1).  Its threads stand for the columns i0-1 .. i0+wout (the band plus one ring
-// column on each side) and sweep the rows j0-1 .. j1 in order.  At row j every thread
-// reconstructs its cell (i, j) once from a 3-row shared-memory window of the stage input;
-// the x-face fluxes of row j are formed once per face through shared memory, the y-face
-// flux between rows j-1 and j is formed by the column's own thread from the top traces it
-// kept from row j-1, and the cell (i, j-1) is then complete: its stage update is written
-// and the wave speed of the output is folded into a block maximum.  Redundant work is the
-// two ring columns per band and the two ring rows per chunk (x pass skipped on ring rows).
+// Decomposition, as in FP64: a block owns a band of wout <= BX-2 output columns and a chunk of
+// output rows [j0, j1).  Its BX x BY threads stand for the columns i0-1 .. i0+wout (the band plus
+// one ring column on each side) of BY consecutive rows, and sweep the rows j0-1 .. j1 BY at a
+// time.  Every thread reconstructs its cell (i, j) once from a (BY + 2)-row shared-memory window
+// of the stage input; the x-face fluxes of a row are formed once per face through shared memory
+// by the row's threads, the y-face fluxes once per face by the threads above the face from the
+// traces below it (those of the tile's last row carried to the next step).  A row is complete
+// once the face above it is (the tile's last row one step later): its stage update is written
+// and the wave speed of the output is folded into a block maximum.  Redundant work is the two
+// ring columns per band and the two ring rows per chunk (x pass skipped on ring rows).
 #pragma once
 #include "geometry.h"
 #include "hweno_device.cuh"
@@ -62,14 +64,14 @@ __device__ __forceinline__ void volume_sum(const KProblem& P, int dir, const R (
 
 // One work item: band `band` (output columns band*wout .. +wout-1) and the output rows
 // [j0, j1) of one stage of one solve, processed by a whole block.
-// smem: dynamic shared memory of smem_bytes2d<EQ, CHAR, R, BW>(); red: 2*(BW/32) doubles.
-// The row window holds the stage input in the bulk precision R (converted once per value
-// when a row is loaded); the FP64 update reads the cell's own averages from global memory
-// when R is float.
+// smem: dynamic shared memory of smem_bytes2d<EQ, CHAR, R, BW>(); red: two doubles per warp.
+// In FP32-bulk the row window holds the stage input in the bulk precision (converted once per
+// value when a row is loaded), and the FP64 update reads the cell's own averages from global
+// memory.
 
-// Shared memory of a block: the 3-row window, the x-face exchange and the top traces carried
-// from row to row (in shared memory rather than in 48 registers: fewer spills, FP32-bulk
-// stages 2 % faster).
+// Shared memory of a block, FP32-bulk: the table of constants, the (BY + 2)-row window, the
+// x-face exchange, the y-face moments and the top traces (in shared memory rather than in
+// registers: fewer spills, stages 2 % faster).
 template <int EQ, bool CHAR, typename R, int BW>
 constexpr size_t smem_bytes2d() {
   constexpr int NC = (EQ == EQ_EULER) ? 4 : 1;

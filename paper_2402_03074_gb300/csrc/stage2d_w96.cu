@@ -1,4 +1,4 @@
-// stage2d_w96.cu -- the 96-thread instantiations of the single-solve 2D stage kernel
+// stage2d_w96.cu -- the 96-column instantiations of the single-solve 2D stage kernel
 // (stage2d_impl.cuh), compiled apart from the other widths.
 #include "stage2d_impl.cuh"
 
