@@ -234,9 +234,9 @@ int hweno_stage_batch_static(int n, const hweno_problem* problems, int k,
 /* Time one fused stage launch of the 2D problem p on a scratch copy of moments_host in the tile
    that a grid without an entry takes (32, 64 or 96 columns, chosen for the grid) and in each
    candidate tile shape -- the block width (128, 96, 64 or 192 columns of threads: a band plus its
-   two ring columns, by one to eight rows) x the number of bands the columns are split into (the default bands,
-   and 1.25, 1.5 and 2 times as many as the widest bands of that width) x the height of the
-   row chunks a block sweeps (the default one-wave geometry and 8, 16, 32, 64, 128, 256 rows)
+   two ring columns, by one to four rows) x the number of bands the columns are split into (the
+   default bands, and 1.25, 1.5 and 2 times as many as the widest bands of that width) x the height
+   of the row chunks a block sweeps (the default one-wave geometry and 8, 16, 32, 64, 128, 256 rows)
    -- then time the closest candidates (at most four, within 3 % of the fastest) again over
    whole three-stage sequences, keep the fastest sequence's shape in the process-wide tuning
    table (keyed by equation, characteristic decomposition, precision and grid) for every
@@ -245,11 +245,11 @@ int hweno_stage_batch_static(int n, const hweno_problem* problems, int k,
    The scratch copy is stepped with dt = 0.  For a 1D problem the
    candidates are the block width (128 or 32 threads) and the threads per cell (one per cell,
    or -- every FP64 problem, and FP32-bulk Euler with the characteristic decomposition -- four
-   lanes per cell in blocks of 128, 64 or 32 threads); *best_rows receives the block width and *best_bands the
-   threads per cell (1 or 4).  Output pointers may be NULL.  The 2D bands, rows and block width
-   change no result bit (every cell and face is computed by the same code in any decomposition),
-   nor do the threads per cell of a 1D problem in FP64; the FP32-bulk 1D layouts compute the same
-   formulas, equal within rounding. */
+   lanes per cell in blocks of 128, 64 or 32 threads); *best_rows receives the block width and
+   *best_bands the threads per cell (1 or 4).  Output pointers may be NULL.  The 2D bands, rows and
+   block width change no result bit (every cell and face is computed by the same code in any
+   decomposition), nor do the threads per cell of a 1D problem in FP64; the FP32-bulk 1D layouts
+   compute the same formulas, equal within rounding. */
 int hweno_autotune(hweno_engine* eng, const hweno_problem* p, const double* moments_host,
                    int* best_rows, int* best_bands, double* best_ms);
 /* Save the tuning table as text (one entry per line, with the GPU name); load it back
@@ -260,9 +260,9 @@ int hweno_tuning_load(const char* path);
    shape; 0 = the default, -1 = the default chosen by the autotuner; rows < -1: the bands'
    rows swept in segments of -rows band-rows, one per block), *width (block width: 2D
    192, 128, 96, 64 or 32, 1D 128, 64 or 32; 0 = the default, and 2D 96 with rows = bands = 0 the
-   autotuner's entry for it: the tile chosen for the grid, 32, 64 or 96 columns) and *lanes (1D threads per cell).  Returns 1
-   when the table has an entry for p, 0 when not (all outputs 0), HWENO_ERR_ARG for a NULL or
-   malformed p.  Output pointers may be NULL. */
+   autotuner's entry for it: the tile chosen for the grid, 32, 64 or 96 columns) and *lanes (1D
+   threads per cell).  Returns 1 when the table has an entry for p, 0 when not (all outputs 0),
+   HWENO_ERR_ARG for a NULL or malformed p.  Output pointers may be NULL. */
 int hweno_tuning_query(const hweno_problem* p, int* rows, int* bands, int* width, int* lanes);
 
 /* ---------------------------------------------------------------------------------------
